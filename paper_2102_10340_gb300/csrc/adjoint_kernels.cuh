@@ -54,15 +54,17 @@ __device__ __forceinline__ T warp_sum_t(T x) {
 // the co-state at time t_hi - s - 1 from the one at t_hi - s, using the state
 // at time t_hi - s - 1 (state.u[s], state.v[s]) at the centre cell.  State
 // rows travel through a per-warp shared-memory ring (one per stage) filled by
-// cp.async in the same commit groups as the co-state rows, kRing - 1 beats
-// ahead of use.  The six gene sums run in T over the owned cells and reach
+// cp.async in the same commit groups as the co-state rows, as many
+// beats ahead of use.  The six gene sums run in T over the owned cells and reach
 // FP64 once per warp (FP64 arithmetic is slow here).
 template <typename T, int K, int RX, int BC>
 struct ReversePolicy {
     // A stage reads only its own ring slot of the beat and sums over owned
     // rows (q >= K, inside the light cone), so the fill may skip stages; the
     // state-row copies are issued per beat for every stage regardless.
-    static constexpr bool kLightCone = true;
+    static constexpr bool kOutputSum = false;  // sums of the co-state itself, for every model
+    static constexpr int V = Vec<T>::N;
+    static constexpr int R = RingRows<StageRows<T, V, K, BC, false>::kPhases>::value;
     typedef typename Vec<T>::type VT;
     const AdjCoef<T> &p;
     const StripGeom &geo;
@@ -70,7 +72,7 @@ struct ReversePolicy {
     T *__restrict__ lun;
     T *__restrict__ lvn;
     int nn, nm;
-    VT (*aux)[kRing][2][32];  // [stage][slot][field][lane]
+    VT (*aux)[R][2][32];  // [stage][slot][field][lane]
     RowWalk<BC> gw[K];        // next state row to copy, per stage (wrapped / reflected)
     T rg[6];                  // sums: u Lap(lu), v Lap(lv), lv, lv v, lv (u - b v), lu u
 
@@ -81,23 +83,20 @@ struct ReversePolicy {
 #pragma unroll
         for (int s = 0; s < K; ++s) gw[s].start((int64_t)geo.r0 - K - s - 1, nn);
     }
-    __device__ __forceinline__ void issue(int j) {
+    __device__ __forceinline__ void issue(int, int slot) {
         const int lane = threadIdx.x & 31;
 #pragma unroll
         for (int s = 0; s < K; ++s) {
             const int64_t off = (int64_t)gw[s].g * nm + geo.lc;
-            cp_async16(&aux[s][j % kRing][0][lane], state.u[s] + off);
-            cp_async16(&aux[s][j % kRing][1][lane], state.v[s] + off);
+            cp_async16(&aux[s][slot][0][lane], state.u[s] + off);
+            cp_async16(&aux[s][slot][1][lane], state.v[s] + off);
             gw[s].next(nn);
         }
     }
-    __device__ __forceinline__ void begin_beat(int) {}
-    __device__ __forceinline__ void stage(int s, const Slice<T> &A, const Slice<T> &B, const Slice<T> &C,
-                                          T wu, T eu, T wv, T ev, int q, Slice<T> &out) {
-        constexpr int V = Vec<T>::N;
+    __device__ __forceinline__ void stage(int s, const Slice<T> &B, const T (&nu)[V], const T (&nv)[V], const T (&)[V],
+                                          int q, int slot, Slice<T> &out) {
         const bool own = (q >= K) && (q < K + geo.nout) && geo.st_lane;
         const int lane = threadIdx.x & 31;
-        const int slot = (q + s + 1) % kRing;  // beat m = q + s + 1
         const VT su4 = aux[s][slot][0][lane];
         const VT sv4 = aux[s][slot][1][lane];
         const T *stu = reinterpret_cast<const T *>(&su4);
@@ -105,10 +104,7 @@ struct ReversePolicy {
 #pragma unroll
         for (int e = 0; e < V; ++e) {
             const T luc = B.u[e], lvc = B.v[e];
-            const T su = add_rn(add_rn(A.u[e], C.u[e]), add_rn(e == 0 ? wu : B.u[e - 1],
-                                                               e == V - 1 ? eu : B.u[e + 1]));
-            const T sv = add_rn(add_rn(A.v[e], C.v[e]), add_rn(e == 0 ? wv : B.v[e - 1],
-                                                               e == V - 1 ? ev : B.v[e + 1]));
+            const T su = nu[e], sv = nv[e];
             // a mirrored lane holds its state vector reversed, like its co-state
             const bool flip = (BC == BC_MIRROR) && geo.rev;
             const T uc = flip ? stu[V - 1 - e] : stu[e];
@@ -195,8 +191,9 @@ k_adjoint_pipe(const T *__restrict__ lu, const T *__restrict__ lv, T *__restrict
     typedef typename Vec<T>::type VT;
     // state rings in dynamic shared memory: [warp][stage][slot][field][lane]
     extern __shared__ __align__(16) unsigned char adj_dyn_smem[];
-    VT(*aux_mem)[K][kRing][2][32] = reinterpret_cast<VT(*)[K][kRing][2][32]>(adj_dyn_smem);
-    ReversePolicy<T, K, RX, BC> pol{p, geo, state, lun, lvn, nn, nm, aux_mem[(threadIdx.x >> 5) % kTemporalWarps]};
+    typedef ReversePolicy<T, K, RX, BC> Pol;
+    VT(*aux_mem)[K][Pol::R][2][32] = reinterpret_cast<VT(*)[K][Pol::R][2][32]>(adj_dyn_smem);
+    Pol pol{p, geo, state, lun, lvn, nn, nm, aux_mem[(threadIdx.x >> 5) % kTemporalWarps]};
     pol.init();
     pipeline_strip<T, K, BC>(geo, lu, lv, nn, nm, pol);
     pol.flush(partial + (int64_t)wid * 6);
@@ -224,9 +221,9 @@ struct PipeShape {
 };
 
 // Dynamic shared memory of k_adjoint_pipe<T, K>: the per-stage state rings.
-template <typename T, int K>
+template <typename T, int K, int BC>
 constexpr size_t pipe_smem_bytes() {
-    return (size_t)kTemporalWarps * K * kRing * 2 * 32 * sizeof(typename Vec<T>::type);
+    return (size_t)kTemporalWarps * K * ReversePolicy<T, K, RX_FHN, BC>::R * 2 * 32 * sizeof(typename Vec<T>::type);
 }
 
 // Opt the kernel in to its dynamic shared memory (above the 48 KB default), once.
@@ -235,7 +232,7 @@ cudaError_t pipe_smem_optin() {
     static cudaError_t done = cudaErrorNotReady;
     if (done == cudaErrorNotReady)
         done = cudaFuncSetAttribute(k_adjoint_pipe<T, K, H, RX, BC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)pipe_smem_bytes<T, K>());
+                                    (int)pipe_smem_bytes<T, K, BC>());
     return done;
 }
 
@@ -246,10 +243,10 @@ cudaError_t reverse_launch_kh(int reaction, int boundary, const void *lu, const 
                               const PipeShape &sh, const rdcnn_params &p, cudaStream_t s) {
     const unsigned grid = (unsigned)((sh.nwarps + kTemporalWarps - 1) / kTemporalWarps);
     const AdjCoef<T> c = make_adj_coef<T>(p, reaction);
-    const size_t smem = pipe_smem_bytes<T, K>();
     return with_model(reaction, boundary, [&](auto rx, auto bc) {
         constexpr int RX = decltype(rx)::value;
         constexpr int BC = decltype(bc)::value;
+        const size_t smem = pipe_smem_bytes<T, K, BC>();
         const cudaError_t oe = pipe_smem_optin<T, K, H, RX, BC>();
         if (oe != cudaSuccess) return oe;
         const cudaError_t e = launch_k(k_adjoint_pipe<T, K, H, RX, BC>, grid, kPipeBlock, smem, s, (const T *)lu,

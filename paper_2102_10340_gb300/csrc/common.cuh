@@ -4,8 +4,8 @@
 // Eq. 2-3, or one of the other local models the simulator is a template for
 // (Sec. I, Sec. II.A): pure diffusion, and the Chua-Yang cellular neural
 // network cell.  Every kernel of the library (single step, temporally
-// blocked, batched) computes a cell through cell_update() below, and
-// cell_update() spells out each rounding with the *_rn intrinsics, so the
+// blocked, batched) computes a cell through nbr_sum() and cell_react() below,
+// which spell out each rounding with the *_rn intrinsics, so the
 // compiler cannot contract or reorder differently in different kernels: all
 // variants give bit-identical states for the same inputs.
 #pragma once
@@ -232,31 +232,40 @@ __device__ __forceinline__ double fma_rn(double x, double y, double z) { return 
 __device__ __forceinline__ float clamp1(float x) { return fminf(fmaxf(x, -1.0f), 1.0f); }
 __device__ __forceinline__ double clamp1(double x) { return fmin(fmax(x, -1.0), 1.0); }
 
-// One cell.  c* = centre, n/s = rows i-1/i+1, w/e = columns j-1/j+1.
+// Sum of the four neighbours of a cell (rows i-1 / i+1, columns j-1 / j+1).
+// On the torus the sum is grouped (n + w) + (s + e): s + e of cell (i, j) is
+// n + w of cell (i+1, j+1), so the pipelines of temporal.cuh form each pair
+// once and spend two additions per cell instead of three, with these bits.
+// Under zero flux the grouping is (n + s) + (w + e), which a reflection about
+// a row or a column leaves unchanged (IEEE addition commutes), as the mirrored
+// halos need.
+template <int BC, typename T>
+__device__ __forceinline__ T nbr_sum(T n, T s, T w, T e) {
+    if constexpr (BC == BC_MIRROR) return add_rn(add_rn(n, s), add_rn(w, e));
+    else return add_rn(add_rn(n, w), add_rn(s, e));
+}
+
+// One cell from its centre and its neighbour sums su, sv.
 // FitzHugh-Nagumo (Eq. 1-3) is evaluated as
-//   u+ = u + dt [ Du ((n + s) + (w + e)) + u (c - 4 Du - u^2/3) - v ]
-//   v+ = v + dt [ Dv ((n + s) + (w + e)) - eps u + (eps b - 4 Dv) v - eps a ]
+//   u+ = u + dt [ Du su + u (c - 4 Du - u^2/3) - v ]
+//   v+ = v + dt [ Dv sv - eps u + (eps b - 4 Dv) v - eps a ]
 // i.e. with the -4 Du u (-4 Dv v) term of the Laplacian moved into the
-// reaction polynomial: 15 FP instructions per cell instead of 18.  The state
+// reaction polynomial: 9 FP instructions besides the sums.  The state
 // is the exact addend of the last FMA, so the FP32 accuracy is that of the
 // literal form.
 // CeNN (Chua-Yang cell, output y(x) = clamp(x, -1, 1), which equals
 // (|x + 1| - |x - 1|) / 2; u = state x, v = offset plane w, held constant):
-//   u+ = u + dt [ Du ((y_n + y_s) + (y_w + y_e)) + c y(u) + (w - u) ],  v+ = v.
+//   u+ = u + dt [ Du su + c y(u) + (w - u) ],  v+ = v,
+// su the sum of the neighbours' outputs, yc the cell's own; sv is unused.
 // A NaN state stays NaN (it is the exact addend); a NaN neighbour's output
 // saturates to -1 instead of propagating.
 template <typename T, int RX>
-__device__ __forceinline__ void cell_update(T uc, T un, T us, T uw, T ue,
-                                            T vc, T vn, T vs, T vw, T ve,
-                                            const Coef<T> &p, T &out_u, T &out_v) {
+__device__ __forceinline__ void cell_react(T uc, T vc, T su, T sv, T yc, const Coef<T> &p, T &out_u, T &out_v) {
     if constexpr (RX == RX_CENN) {
-        const T sy = add_rn(add_rn(clamp1(un), clamp1(us)), add_rn(clamp1(uw), clamp1(ue)));
-        out_u = fma_rn(p.dt, fma_rn(p.Du, sy, fma_rn(p.cm4, clamp1(uc), add_rn(vc, -uc))), uc);
+        out_u = fma_rn(p.dt, fma_rn(p.Du, su, fma_rn(p.cm4, yc, add_rn(vc, -uc))), uc);
         out_v = vc;
         return;
     }
-    const T su = add_rn(add_rn(un, us), add_rn(uw, ue));      // neighbour sum of u
-    const T sv = add_rn(add_rn(vn, vs), add_rn(vw, ve));      // neighbour sum of v
     T ru, rv;
     if (RX == RX_FHN) {
         const T cm = fma_rn(mul_rn(uc, uc), p.mthird, p.cm4);  // c - 4 Du - u^2/3
@@ -268,6 +277,20 @@ __device__ __forceinline__ void cell_update(T uc, T un, T us, T uw, T ue,
     }
     out_u = fma_rn(p.dt, fma_rn(p.Du, su, ru), uc);
     out_v = fma_rn(p.dt, fma_rn(p.Dv, sv, rv), vc);
+}
+
+// One cell from its five-point neighbourhood.  c* = centre, n/s = rows
+// i-1/i+1, w/e = columns j-1/j+1.
+template <typename T, int RX, int BC>
+__device__ __forceinline__ void cell_update(T uc, T un, T us, T uw, T ue,
+                                            T vc, T vn, T vs, T vw, T ve,
+                                            const Coef<T> &p, T &out_u, T &out_v) {
+    if constexpr (RX == RX_CENN) {
+        const T sy = nbr_sum<BC>(clamp1(un), clamp1(us), clamp1(uw), clamp1(ue));
+        cell_react<T, RX>(uc, vc, sy, T(0), clamp1(uc), p, out_u, out_v);
+    } else {
+        cell_react<T, RX>(uc, vc, nbr_sum<BC>(un, us, uw, ue), nbr_sum<BC>(vn, vs, vw, ve), T(0), p, out_u, out_v);
+    }
 }
 
 // A lane's slice of one grid row for both fields: V consecutive columns.
@@ -293,7 +316,7 @@ __device__ __forceinline__ void store_vec(T *__restrict__ dst, const CT<T> (&src
 // The west neighbour of element 0 and the east neighbour of element V-1 come
 // from the adjacent lanes (or, for lanes whose neighbour is not in the warp,
 // from the caller: west_u/east_u etc.).
-template <typename T, int RX, int V = Vec<T>::N>
+template <typename T, int RX, int BC, int V = Vec<T>::N>
 __device__ __forceinline__ void slice_update(const Slice<T, V> &nor, const Slice<T, V> &cen,
                                              const Slice<T, V> &sou, T west_u, T east_u,
                                              T west_v, T east_v, const Coef<T> &p,
@@ -304,9 +327,19 @@ __device__ __forceinline__ void slice_update(const Slice<T, V> &nor, const Slice
         const T eu = (e == V - 1) ? east_u : cen.u[e + 1];
         const T wv = (e == 0) ? west_v : cen.v[e - 1];
         const T ev = (e == V - 1) ? east_v : cen.v[e + 1];
-        cell_update<T, RX>(cen.u[e], nor.u[e], sou.u[e], wu, eu,
+        cell_update<T, RX, BC>(cen.u[e], nor.u[e], sou.u[e], wu, eu,
                         cen.v[e], nor.v[e], sou.v[e], wv, ev, p, out.u[e], out.v[e]);
     }
+}
+
+// The same from neighbour sums formed by the caller (temporal.cuh: StageRows).
+template <typename T, int RX, int V = Vec<T>::N>
+__device__ __forceinline__ void slice_react(const Slice<T, V> &cen, const T (&su)[V], const T (&sv)[V],
+                                            const T (&yc)[V], const Coef<T> &p, Slice<T, V> &out) {
+#pragma unroll
+    for (int e = 0; e < V; ++e)
+        cell_react<T, RX>(cen.u[e], cen.v[e], su[e], RX == RX_CENN ? T(0) : sv[e], RX == RX_CENN ? yc[e] : T(0), p,
+                          out.u[e], out.v[e]);
 }
 
 template <typename T>

@@ -20,7 +20,7 @@
 //              values after K steps and do not store.
 //  k_generic   one thread per cell, scalar loads: any size and alignment.
 //
-// All three evaluate cells with rdk::cell_update, so they produce identical
+// All three evaluate cells with rdk::nbr_sum and rdk::cell_react, so they produce identical
 // bits for identical inputs (for 16-bit planes: at the same steps per
 // launch, which is also the rounding interval).  Under the zero-flux boundary the single-step
 // and generic kernels clamp neighbour indices into the grid (the ghost cell
@@ -115,7 +115,7 @@ k_step1(const T *__restrict__ u, const T *__restrict__ v, T *__restrict__ un,
         if (edge_w) { wu = cw_u; wv = cw_v; }
         if (edge_e) { eu = ce_u; ev = ce_v; }
         Slice<T> out;
-        slice_update<T, RX>(nor, cen, sou, wu, eu, wv, ev, p, out);
+        slice_update<T, RX, BC>(nor, cen, sou, wu, eu, wv, ev, p, out);
         if (active) {
             const int64_t off = (int64_t)r * nm + col;
             store_vec<T>(un + off, out.u);
@@ -152,7 +152,7 @@ k_generic(const T *__restrict__ u, const T *__restrict__ v, T *__restrict__ un,
         const int64_t rp = (int64_t)ip * nm;
         const int64_t rm = (int64_t)im * nm;
         CT<T> ou, ov;
-        cell_update<CT<T>, RX>(load1(u + ri + j), load1(u + rm + j), load1(u + rp + j), load1(u + ri + jm),
+        cell_update<CT<T>, RX, BC>(load1(u + ri + j), load1(u + rm + j), load1(u + rp + j), load1(u + ri + jm),
                                load1(u + ri + jp), load1(v + ri + j), load1(v + rm + j), load1(v + rp + j),
                                load1(v + ri + jm), load1(v + ri + jp), p, ou, ov);
         un[idx] = to_storage<T>(ou);

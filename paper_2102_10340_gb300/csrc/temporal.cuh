@@ -6,7 +6,7 @@
 // of an NN x NM torus.  It loads 32*V columns starting H*V columns to the left
 // of its band (H = ceil(K/V) halo lanes per side, indices wrapped modulo NM)
 // and input rows r0-K .. r0+rows+K-1 (wrapped modulo NN).  Input rows are
-// staged through a per-warp shared-memory ring by cp.async, kRing - 1 rows
+// staged through a per-warp shared-memory ring by cp.async, two or three rows
 // ahead of use.  Each input row passes through K stages held in registers;
 // stage s turns rows (q-1, q, q+1)
 // of stage s-1 into row q of stage s.  After K stages the K outermost columns
@@ -35,10 +35,13 @@ namespace rdk {
 // 0.44 to 0.18 and issue-active rising from 63 % to 72 % at the same 8
 // warps per SM and the same instructions).
 constexpr int kTemporalWarps = 1;
-// Input rows staged per warp (prefetch distance kRing - 1 = 2 beats, about
-// 1.5 us of the K = 8 pipeline, above the HBM latency).  Three slots match
-// the 3-beat window rotation, so a beat's slots are compile-time constants.
+// Input rows staged per warp by the three-phase pipelines (prefetch distance
+// kRing - 1 = 2 beats, about 1.5 us of the K = 8 pipeline, above the HBM
+// latency).  Three slots match the 3-beat window rotation, so a beat's slots
+// are compile-time constants.  The two-phase pipelines keep kRing2 rows (a
+// power of two; the slot of a beat is a running index).
 constexpr int kRing = 3;
+constexpr int kRing2 = 4;
 
 // Per-lane 16-byte asynchronous global -> shared copy (cp.async, L2 only).
 __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
@@ -54,12 +57,12 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
-// Shared-memory ring of one warp: kRing rows x {u, v} x 32 lanes x 16 bytes.
+// Shared-memory ring of one warp: rows x {u, v} x 32 lanes x 16 bytes.
 // Each lane copies and later reads back only its own 16 bytes, so the lane's
 // own cp.async.wait_group is the only synchronisation needed.
 template <typename T> struct RowRing {
     typedef typename Vec<T>::type VT;
-    VT (*slot)[2][32];  // [kRing][field][lane]
+    VT (*slot)[2][32];  // [row][field][lane]
 };
 
 template <typename T>
@@ -148,69 +151,208 @@ template <int BC> struct RowWalk {
     }
 };
 
-// One pipeline beat: take input row m of the strip from the ring (issuing the
-// copy of row m + kRing - 1 first), advance every stage by one row, and hand
-// the finished row (stage K) to the policy.  W[PH], W[PH+1] hold the two older
-// rows of each stage, W[PH+2] receives the newest, so a 3-beat unroll rotates
-// the windows without register moves.
+// The rows one stage keeps between beats, and the neighbour sums they give.
+// cen = row q of the stage's input, C = row q + 1, just arrived.
+//
+// Torus, linear sums: the cell sum is (n + w) + (s + e), and s + e of cell
+// (q, j) is n + w of cell (q + 1, j + 1).  So a stage keeps row q and the
+// pair sums acc(j) = row_{q-1}(j+1) + row_q(j) instead of rows q - 1 and q:
+// the sum of a cell is its own new pair (row_q(j+1) + C(j)) plus the old pair
+// one column to the west -- two additions per field instead of three, at the
+// same registers and the same two shuffles.  4096^2, K = 8: @PAIR@
+// Zero flux: rows q - 1 and q, three additions (nbr_sum says why).
+// CeNN cell (OUT): the sums run over the outputs y = clamp(x), clamped once
+// when a row arrives and kept (pair sums and y of row q on the torus, y of
+// rows q - 1 and q under zero flux) instead of once per neighbour; v is
+// constant, so it needs no sums.  4096^2, K = 8: torus 73.5 -> 57.2 us a
+// launch, zero flux 75.7 -> 69.6 us.
+//
+// Row sets rotate by beat phase PH = m % kPhases without register moves:
+// two-phase stages hold row q in row[PH] and put C into row[PH ^ 1], the
+// three-phase ones hold rows q - 1, q, q + 1 in row[PH], row[PH + 1],
+// row[PH + 2].
+template <typename T, int V, int K, int BC, bool OUT> struct StageRows {
+    static constexpr bool kPair = (BC == BC_WRAP && K > 1);
+    static constexpr int kPhases = (!kPair && !OUT) ? 3 : 2;
+    Slice<T, V> row[kPhases];
+    T acc[2][V];
+
+    __device__ __forceinline__ void zero() {
+#pragma unroll
+        for (int a = 0; a < kPhases; ++a) zero_slice(row[a]);
+#pragma unroll
+        for (int e = 0; e < V; ++e) acc[0][e] = acc[1][e] = T(0);
+    }
+
+    template <int PH>
+    __device__ __forceinline__ const Slice<T, V> &cen() const {
+        return kPhases == 3 ? row[(PH + 1) % 3] : row[PH];
+    }
+    template <int PH>
+    __device__ __forceinline__ void put(const Slice<T, V> &C) {
+        row[kPhases == 3 ? (PH + 2) % 3 : (PH ^ 1)] = C;
+    }
+
+    // Take in a row without computing one (light-cone fill): the stage's
+    // first row, or (FIRST = false) its second.
+    template <int PH, bool FIRST>
+    __device__ __forceinline__ void keep(const Slice<T, V> &C) {
+        if constexpr (kPhases == 2) {
+            const Slice<T, V> &B = row[PH];
+            if constexpr (!OUT) {
+                if constexpr (!FIRST) {  // (linear two-phase stages keep pairs)
+                    const T eu = __shfl_down_sync(kFull, B.u[0], 1);
+                    const T ev = __shfl_down_sync(kFull, B.v[0], 1);
+#pragma unroll
+                    for (int e = 0; e < V; ++e) {
+                        acc[0][e] = add_rn(e == V - 1 ? eu : B.u[e + 1], C.u[e]);
+                        acc[1][e] = add_rn(e == V - 1 ? ev : B.v[e + 1], C.v[e]);
+                    }
+                }
+            } else if constexpr (kPair) {
+                T y[V];
+#pragma unroll
+                for (int e = 0; e < V; ++e) y[e] = clamp1(C.u[e]);
+                if constexpr (!FIRST) {
+                    const T ey = __shfl_down_sync(kFull, acc[1][0], 1);
+#pragma unroll
+                    for (int e = 0; e < V; ++e) acc[0][e] = add_rn(e == V - 1 ? ey : acc[1][e + 1], y[e]);
+                }
+#pragma unroll
+                for (int e = 0; e < V; ++e) acc[1][e] = y[e];
+            } else {  // outputs of rows q - 1, q in acc[PH], acc[PH ^ 1]
+#pragma unroll
+                for (int e = 0; e < V; ++e) acc[PH][e] = clamp1(C.u[e]);
+            }
+        }
+        put<PH>(C);
+    }
+
+    // The neighbour sums su, sv (and the outputs yc, OUT only) of row q; then
+    // C takes its place among the kept rows (the caller calls put<PH>(C)).
+    template <int PH>
+    __device__ __forceinline__ void sums(const Slice<T, V> &C, T (&su)[V], T (&sv)[V], T (&yc)[V]) {
+        const Slice<T, V> &B = cen<PH>();
+        if constexpr (OUT) {
+            T y[V];
+#pragma unroll
+            for (int e = 0; e < V; ++e) y[e] = clamp1(C.u[e]);
+            if constexpr (kPair) {
+                const T wy = __shfl_up_sync(kFull, acc[0][V - 1], 1);
+                const T ey = __shfl_down_sync(kFull, acc[1][0], 1);
+#pragma unroll
+                for (int e = V - 1; e >= 0; --e) {
+                    const T a = add_rn(e == V - 1 ? ey : acc[1][e + 1], y[e]);
+                    su[e] = add_rn(e == 0 ? wy : acc[0][e - 1], a);
+                    acc[0][e] = a;
+                }
+#pragma unroll
+                for (int e = 0; e < V; ++e) {
+                    yc[e] = acc[1][e];
+                    acc[1][e] = y[e];
+                }
+            } else {
+                const T wy = __shfl_up_sync(kFull, acc[PH ^ 1][V - 1], 1);
+                const T ey = __shfl_down_sync(kFull, acc[PH ^ 1][0], 1);
+#pragma unroll
+                for (int e = 0; e < V; ++e) {
+                    su[e] = nbr_sum<BC>(acc[PH][e], y[e], e == 0 ? wy : acc[PH ^ 1][e - 1],
+                                        e == V - 1 ? ey : acc[PH ^ 1][e + 1]);
+                    yc[e] = acc[PH ^ 1][e];
+                }
+#pragma unroll
+                for (int e = 0; e < V; ++e) acc[PH][e] = y[e];
+            }
+        } else if constexpr (kPair) {
+            const T wu = __shfl_up_sync(kFull, acc[0][V - 1], 1);
+            const T eu = __shfl_down_sync(kFull, B.u[0], 1);
+            const T wv = __shfl_up_sync(kFull, acc[1][V - 1], 1);
+            const T ev = __shfl_down_sync(kFull, B.v[0], 1);
+#pragma unroll
+            for (int e = V - 1; e >= 0; --e) {
+                const T a = add_rn(e == V - 1 ? eu : B.u[e + 1], C.u[e]);
+                const T b = add_rn(e == V - 1 ? ev : B.v[e + 1], C.v[e]);
+                su[e] = add_rn(e == 0 ? wu : acc[0][e - 1], a);
+                sv[e] = add_rn(e == 0 ? wv : acc[1][e - 1], b);
+                acc[0][e] = a;
+                acc[1][e] = b;
+            }
+        } else {
+            const Slice<T, V> &A = row[PH];
+            const T wu = __shfl_up_sync(kFull, B.u[V - 1], 1);
+            const T eu = __shfl_down_sync(kFull, B.u[0], 1);
+            const T wv = __shfl_up_sync(kFull, B.v[V - 1], 1);
+            const T ev = __shfl_down_sync(kFull, B.v[0], 1);
+#pragma unroll
+            for (int e = 0; e < V; ++e) {
+                su[e] = nbr_sum<BC>(A.u[e], C.u[e], e == 0 ? wu : B.u[e - 1], e == V - 1 ? eu : B.u[e + 1]);
+                sv[e] = nbr_sum<BC>(A.v[e], C.v[e], e == 0 ? wv : B.v[e - 1], e == V - 1 ? ev : B.v[e + 1]);
+            }
+        }
+    }
+};
+
+// Ring rows of a pipeline with the given number of phases.
+template <int PHASES> struct RingRows : IntC<PHASES == 3 ? kRing : kRing2> {};
+
+// One pipeline beat: take input row m of the strip from ring slot rd (issuing
+// the copy of row m + R - 1 into slot wr first, R the ring's rows), advance
+// every stage by one row, and hand the finished row (stage K) to the policy.
 //
 // The policy P supplies the per-stage arithmetic and the stores:
-//   P::issue(j)                          extra cp.async copies for beat j,
+//   P::kOutputSum                        neighbour sums over clamp(x) (CeNN)
+//   P::issue(j, slot)                    extra cp.async copies for beat j,
 //                                        committed with input row j
-//   P::begin_beat(m)                     before the stages of beat m
-//   P::stage<s>(A, B, C, wu, eu, wv, ev, q, out)
-//        stage s maps rows q-1 (A), q (B), q+1 (C) of its input to row q of
-//        its output (q = input-row index within the strip, see temporal_strip)
+//   P::stage(s, cen, su, sv, yc, q, slot, out)
+//        stage s maps row q (cen) of its input and its neighbour sums to row
+//        q of its output (q = input-row index within the strip, see
+//        temporal_strip); slot = the beat's ring slot
 //   P::finish(q, out)                    the row q leaving the last stage
 //   P::finish_main(q, out)               the same for a beat of the main loop,
 //                                        where q >= K holds: the owned row
 //                                        check may be dropped
 //
-// CHECK = false: a beat of the main loop's whole triplets (m + 2 < total),
+// CHECK = false: a beat of the main loop's whole groups of kPhases beats,
 // which needs neither the end-of-strip test nor the last-copy test (measured
-// at K = 8, 4096^2: 1427 -> 1448 Gcell-updates/s).
+// at K = 8, 4096^2: 1427 -> 1448 Gcell-updates/s); the copies past the strip's
+// last row are of wrapped rows of the grid and are not read.
 //
-// ACTIVE < K (the first 2K beats of a strip with a policy that allows it):
-// only stages s < ACTIVE compute; stage ACTIVE just keeps its input row for
-// the next beats.  Row q of the last stage needs stage s's rows from
-// q - (K - 1 - s) on, and the stored rows have q >= K, so stage s's rows
-// 0 .. s feed nothing that is stored.  Beat m computes stage s's row
-// m - s - 1, so stage s first matters at beat 2s + 2: ACTIVE = m / 2.
-template <typename T, int K, int PH, int BC, int ACTIVE = K, bool CHECK = true, class P>
-__device__ __forceinline__ void pipeline_beat(int m, int total, Slice<CT<T>, Vec<T>::N> (&W)[3][K],
-                                              const RowRing<T> &ring, RowWalk<BC> &walk, int nn, int nm,
-                                              int lc, bool rev, const T *__restrict__ u,
-                                              const T *__restrict__ v, P &pol) {
+// ACTIVE < K (the first 2K beats of a strip): only stages s < ACTIVE compute;
+// stage ACTIVE just keeps its input row for the next beats.  Row q of the
+// last stage needs stage s's rows from q - (K - 1 - s) on, and the stored
+// rows have q >= K, so stage s's rows 0 .. s feed nothing that is stored.
+// Beat m computes stage s's row m - s - 1, so stage s first matters at beat
+// 2s + 2: ACTIVE = m / 2, and stage ACTIVE keeps its first row at beat 2s and
+// its second at beat 2s + 1.
+template <typename T, int K, int PH, int BC, int ACTIVE = K, bool CHECK = true, bool FIRST = false, class S, class P>
+__device__ __forceinline__ void pipeline_beat(int m, int total, S (&st)[K], const RowRing<T> &ring, int rd, int wr,
+                                              RowWalk<BC> &walk, int nn, int nm, int lc, bool rev,
+                                              const T *__restrict__ u, const T *__restrict__ v, P &pol) {
     constexpr int V = Vec<T>::N;
+    constexpr int R = RingRows<S::kPhases>::value;
     if (CHECK && m >= total) return;
     // The slot written here was read in the previous beat, whose stage
     // computations (issued before this point) consumed that value.
-    static_assert(kRing == 3, "slots follow the 3-beat phase: row m sits in slot m % 3 == PH");
-    if (!CHECK || m + kRing - 1 < total) {
-        ring_issue_at(ring, (PH + kRing - 1) % kRing, walk.g, nm, lc, u, v);
+    if (!CHECK || m + R - 1 < total) {
+        ring_issue_at(ring, wr, walk.g, nm, lc, u, v);
         walk.next(nn);
-        pol.issue(m + kRing - 1);
+        pol.issue(m + R - 1, wr);
     }
     cp_async_commit();
-    cp_async_wait<kRing - 1>();  // the group holding row m is complete
-    Slice<CT<T>, Vec<T>::N> cur;
-    ring_read_bc<T, BC>(ring, PH, rev, cur);
-    pol.begin_beat(m);
+    cp_async_wait<R - 1>();  // the group holding row m is complete
+    Slice<CT<T>, V> cur;
+    ring_read_bc<T, BC>(ring, rd, rev, cur);
 #pragma unroll
     for (int s = 0; s < K; ++s) {
         if (s < ACTIVE) {
-            Slice<CT<T>, Vec<T>::N> &A = W[PH][s];
-            Slice<CT<T>, Vec<T>::N> &B = W[(PH + 1) % 3][s];
-            const CT<T> wu = __shfl_up_sync(kFull, B.u[V - 1], 1);
-            const CT<T> eu = __shfl_down_sync(kFull, B.u[0], 1);
-            const CT<T> wv = __shfl_up_sync(kFull, B.v[V - 1], 1);
-            const CT<T> ev = __shfl_down_sync(kFull, B.v[0], 1);
-            Slice<CT<T>, Vec<T>::N> out;
-            pol.stage(s, A, B, cur, wu, eu, wv, ev, m - s - 1, out);
-            W[(PH + 2) % 3][s] = cur;
+            CT<T> su[V], sv[V], yc[V];
+            st[s].template sums<PH>(cur, su, sv, yc);
+            Slice<CT<T>, V> out;
+            pol.stage(s, st[s].template cen<PH>(), su, sv, yc, m - s - 1, rd, out);
+            st[s].template put<PH>(cur);
             cur = out;
         } else if (s == ACTIVE) {
-            W[(PH + 2) % 3][s] = cur;  // stage s - 1's row, needed from the next beat on
+            st[s].template keep<PH, FIRST>(cur);  // stage s - 1's row, needed from the next beat on
         }
     }
     if constexpr (ACTIVE == K) {
@@ -220,14 +362,15 @@ __device__ __forceinline__ void pipeline_beat(int m, int total, Slice<CT<T>, Vec
 }
 
 // The first 2K beats of a strip (ACTIVE = M / 2), unrolled at compile time.
-template <typename T, int K, int BC, int M, class P>
-__device__ __forceinline__ void pipeline_fill(int total, Slice<CT<T>, Vec<T>::N> (&W)[3][K],
-                                              const RowRing<T> &ring, RowWalk<BC> &walk, int nn, int nm,
-                                              int lc, bool rev, const T *__restrict__ u,
+template <typename T, int K, int BC, int M, class S, class P>
+__device__ __forceinline__ void pipeline_fill(int total, S (&st)[K], const RowRing<T> &ring, RowWalk<BC> &walk,
+                                              int nn, int nm, int lc, bool rev, const T *__restrict__ u,
                                               const T *__restrict__ v, P &pol) {
-    pipeline_beat<T, K, M % 3, BC, (M / 2 < K ? M / 2 : K)>(M, total, W, ring, walk, nn, nm, lc, rev, u, v, pol);
+    constexpr int R = RingRows<S::kPhases>::value;
+    pipeline_beat<T, K, M % S::kPhases, BC, (M / 2 < K ? M / 2 : K), true, M % 2 == 0>(
+        M, total, st, ring, M % R, (M + R - 1) % R, walk, nn, nm, lc, rev, u, v, pol);
     if constexpr (M + 1 < 2 * K)
-        pipeline_fill<T, K, BC, M + 1>(total, W, ring, walk, nn, nm, lc, rev, u, v, pol);
+        pipeline_fill<T, K, BC, M + 1>(total, st, ring, walk, nn, nm, lc, rev, u, v, pol);
 }
 
 // Geometry of one (band, strip) work item for depth K and halo H.
@@ -270,66 +413,83 @@ __device__ __forceinline__ StripGeom strip_geom(int band, int strip, int nn, int
 
 // Run one work item through the K-stage pipeline: input rows of (u, v) pass
 // through the stages; the policy decides what each stage computes and stores.
+// Every policy stores (or sums over) owned rows only, q >= K, so the first 2K
+// beats skip the stages outside their light cone.
 template <typename T, int K, int BC = BC_WRAP, class P>
 __device__ __forceinline__ void pipeline_strip(const StripGeom &geo, const T *__restrict__ u,
                                                const T *__restrict__ v, int nn, int nm, P &pol) {
-    Slice<CT<T>, Vec<T>::N> W[3][K];
+    typedef StageRows<CT<T>, Vec<T>::N, K, BC, P::kOutputSum> S;
+    constexpr int N = S::kPhases;
+    constexpr int R = RingRows<N>::value;
+    S st[K];
 #pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int s = 0; s < K; ++s) zero_slice(W[a][s]);
+    for (int s = 0; s < K; ++s) st[s].zero();
 
     typedef typename Vec<T>::type VT;
-    __shared__ __align__(16) VT ring_mem[kTemporalWarps][kRing][2][32];
+    __shared__ __align__(16) VT ring_mem[kTemporalWarps][R][2][32];
     RowRing<T> ring;
     ring.slot = ring_mem[(threadIdx.x >> 5) % kTemporalWarps];
 
-    // prologue: rows 0 .. kRing-2 in flight, one commit group each
+    // prologue: rows 0 .. R-2 in flight, one commit group each
     RowWalk<BC> walk;
     walk.start((int64_t)geo.r0 - K, nn);
 #pragma unroll
-    for (int j = 0; j < kRing - 1; ++j) {
+    for (int j = 0; j < R - 1; ++j) {
         if (j < geo.total) {
-            ring_issue(ring, j, walk.g, nm, geo.lc, u, v);
+            ring_issue_at(ring, j, walk.g, nm, geo.lc, u, v);
             walk.next(nn);
-            pol.issue(j);
+            pol.issue(j, j);
         }
         cp_async_commit();
     }
     // a strip has total = nout + 2K > 2K beats, so the fill always completes
-    constexpr int M0 = P::kLightCone ? 2 * K : 0;
-    if constexpr (P::kLightCone)
-        pipeline_fill<T, K, BC, 0>(geo.total, W, ring, walk, nn, nm, geo.lc, geo.rev, u, v, pol);
+    constexpr int M0 = 2 * K;
+    pipeline_fill<T, K, BC, 0>(geo.total, st, ring, walk, nn, nm, geo.lc, geo.rev, u, v, pol);
     int m = M0;
-    for (; m + 2 < geo.total; m += 3) {  // whole triplets: no per-beat bounds tests
-        pipeline_beat<T, K, M0 % 3, BC, K, false>(m, geo.total, W, ring, walk, nn, nm, geo.lc, geo.rev, u, v, pol);
-        pipeline_beat<T, K, (M0 + 1) % 3, BC, K, false>(m + 1, geo.total, W, ring, walk, nn, nm, geo.lc, geo.rev, u, v,
-                                                         pol);
-        pipeline_beat<T, K, (M0 + 2) % 3, BC, K, false>(m + 2, geo.total, W, ring, walk, nn, nm, geo.lc, geo.rev, u, v,
-                                                         pol);
+    if constexpr (N == 3) {
+        for (; m + 2 < geo.total; m += 3) {  // whole triplets: no per-beat bounds tests
+            pipeline_beat<T, K, M0 % 3, BC, K, false>(m, geo.total, st, ring, M0 % 3, (M0 + 2) % 3, walk, nn, nm,
+                                                      geo.lc, geo.rev, u, v, pol);
+            pipeline_beat<T, K, (M0 + 1) % 3, BC, K, false>(m + 1, geo.total, st, ring, (M0 + 1) % 3, M0 % 3, walk,
+                                                            nn, nm, geo.lc, geo.rev, u, v, pol);
+            pipeline_beat<T, K, (M0 + 2) % 3, BC, K, false>(m + 2, geo.total, st, ring, (M0 + 2) % 3, (M0 + 1) % 3,
+                                                            walk, nn, nm, geo.lc, geo.rev, u, v, pol);
+        }
+        // the last 0 .. 2 beats
+        pipeline_beat<T, K, M0 % 3, BC>(m, geo.total, st, ring, M0 % 3, (M0 + 2) % 3, walk, nn, nm, geo.lc, geo.rev, u,
+                                        v, pol);
+        pipeline_beat<T, K, (M0 + 1) % 3, BC>(m + 1, geo.total, st, ring, (M0 + 1) % 3, M0 % 3, walk, nn, nm, geo.lc,
+                                              geo.rev, u, v, pol);
+    } else {
+        int rd = M0 % R;  // even; row m sits in slot m % R
+        for (; m + 1 < geo.total; m += 2) {  // whole pairs: no per-beat bounds tests
+            pipeline_beat<T, K, 0, BC, K, false>(m, geo.total, st, ring, rd, (rd + R - 1) % R, walk, nn, nm, geo.lc,
+                                                 geo.rev, u, v, pol);
+            pipeline_beat<T, K, 1, BC, K, false>(m + 1, geo.total, st, ring, rd + 1, rd, walk, nn, nm, geo.lc, geo.rev,
+                                                 u, v, pol);
+            rd = (rd + 2) % R;
+        }
+        // the last 0 or 1 beats
+        pipeline_beat<T, K, 0, BC>(m, geo.total, st, ring, rd, (rd + R - 1) % R, walk, nn, nm, geo.lc, geo.rev, u, v,
+                                   pol);
     }
-    // the last 0 .. 2 beats
-    pipeline_beat<T, K, M0 % 3>(m, geo.total, W, ring, walk, nn, nm, geo.lc, geo.rev, u, v, pol);
-    pipeline_beat<T, K, (M0 + 1) % 3>(m + 1, geo.total, W, ring, walk, nn, nm, geo.lc, geo.rev, u, v, pol);
     cp_async_wait<0>();
 }
 
 // Forward policy: Eq. 1 at every stage; the last stage's owned rows are stored.
-// Only owned rows are stored, so the fill may skip the stages outside their
-// light cone (kLightCone).
 template <typename T, int K, int RX>
 struct ForwardPolicy {
-    static constexpr bool kLightCone = true;
+    static constexpr bool kOutputSum = (RX == RX_CENN);
     const Coef<CT<T>> &p;
     const StripGeom &geo;
     T *__restrict__ un;
     T *__restrict__ vn;
     int nm;
-    __device__ __forceinline__ void issue(int) {}
-    __device__ __forceinline__ void begin_beat(int) {}
-    __device__ __forceinline__ void stage(int, const Slice<CT<T>, Vec<T>::N> &A, const Slice<CT<T>, Vec<T>::N> &B, const Slice<CT<T>, Vec<T>::N> &C,
-                                          CT<T> wu, CT<T> eu, CT<T> wv, CT<T> ev, int, Slice<CT<T>, Vec<T>::N> &out) {
-        slice_update<CT<T>, RX, Vec<T>::N>(A, B, C, wu, eu, wv, ev, p, out);
+    __device__ __forceinline__ void issue(int, int) {}
+    __device__ __forceinline__ void stage(int, const Slice<CT<T>, Vec<T>::N> &cen, const CT<T> (&su)[Vec<T>::N],
+                                          const CT<T> (&sv)[Vec<T>::N], const CT<T> (&yc)[Vec<T>::N], int, int,
+                                          Slice<CT<T>, Vec<T>::N> &out) {
+        slice_react<CT<T>, RX, Vec<T>::N>(cen, su, sv, yc, p, out);
     }
     __device__ __forceinline__ void finish(int q, const Slice<CT<T>, Vec<T>::N> &out) {
         const int orow = q - K;
@@ -361,16 +521,16 @@ template <typename T> struct StagePlanes {
 // needs, K per launch.
 template <typename T, int K, int RX>
 struct ForwardAllPolicy {
-    static constexpr bool kLightCone = true;  // stores owned rows only (q >= K)
+    static constexpr bool kOutputSum = (RX == RX_CENN);
     const Coef<CT<T>> &p;
     const StripGeom &geo;
     const StagePlanes<T> &planes;
     int nm;
-    __device__ __forceinline__ void issue(int) {}
-    __device__ __forceinline__ void begin_beat(int) {}
-    __device__ __forceinline__ void stage(int s, const Slice<CT<T>, Vec<T>::N> &A, const Slice<CT<T>, Vec<T>::N> &B, const Slice<CT<T>, Vec<T>::N> &C,
-                                          CT<T> wu, CT<T> eu, CT<T> wv, CT<T> ev, int q, Slice<CT<T>, Vec<T>::N> &out) {
-        slice_update<CT<T>, RX, Vec<T>::N>(A, B, C, wu, eu, wv, ev, p, out);
+    __device__ __forceinline__ void issue(int, int) {}
+    __device__ __forceinline__ void stage(int s, const Slice<CT<T>, Vec<T>::N> &cen, const CT<T> (&su)[Vec<T>::N],
+                                          const CT<T> (&sv)[Vec<T>::N], const CT<T> (&yc)[Vec<T>::N], int q, int,
+                                          Slice<CT<T>, Vec<T>::N> &out) {
+        slice_react<CT<T>, RX, Vec<T>::N>(cen, su, sv, yc, p, out);
         const int orow = q - K;
         if (orow >= 0 && orow < geo.nout && geo.st_lane) {
             const int64_t off = (int64_t)(geo.r0 + orow) * nm + geo.sc;

@@ -78,7 +78,7 @@ __device__ __forceinline__ void split_producer_beat(int m, int total, Slice<T> (
                 const T wv = __shfl_up_sync(kFull, B.v[V - 1], 1);
                 const T ev = __shfl_down_sync(kFull, B.v[0], 1);
                 Slice<T> out;
-                slice_update<T, RX>(A, B, cur, wu, eu, wv, ev, p, out);
+                slice_update<T, RX, BC>(A, B, cur, wu, eu, wv, ev, p, out);
                 W[(PH + 2) % 3][s] = cur;
                 cur = out;
             } else if (s == ACT) {
@@ -101,7 +101,7 @@ __device__ __forceinline__ void split_producer_beat(int m, int total, Slice<T> (
 
 // Consumer beat: the producer's row of beat m - 1 through stages K1+1 .. K; the
 // final row (input-row index m - 1 - K) is stored when the strip owns it.
-template <typename T, int K, int K2, int RX, int PH, int ACT = K2, bool KEEP = false>
+template <typename T, int K, int K2, int RX, int BC, int PH, int ACT = K2, bool KEEP = false>
 __device__ __forceinline__ void split_consumer_beat(int m, int total, Slice<T> (&W)[3][K2],
                                                     const Handoff<T> &hand, const StripGeom &geo,
                                                     T *__restrict__ un, T *__restrict__ vn, int nm,
@@ -121,7 +121,7 @@ __device__ __forceinline__ void split_consumer_beat(int m, int total, Slice<T> (
                 const T wv = __shfl_up_sync(kFull, B.v[V - 1], 1);
                 const T ev = __shfl_down_sync(kFull, B.v[0], 1);
                 Slice<T> out;
-                slice_update<T, RX>(A, B, cur, wu, eu, wv, ev, p, out);
+                slice_update<T, RX, BC>(A, B, cur, wu, eu, wv, ev, p, out);
                 W[(PH + 2) % 3][s] = cur;
                 cur = out;
             } else if (KEEP && s == ACT) {
@@ -153,16 +153,16 @@ __device__ __forceinline__ void split_producer_fill(int total, Slice<T> (&W)[3][
 // Fill beats 0 .. F-1 of the consumer (equivalent beat M - 1): local stage j
 // computes when M - 1 >= 2 (K1 + j) + 2; the next one keeps its input once
 // the handoff row is valid (M - 1 >= 2 K1).
-template <typename T, int K, int K2, int RX, int M, int F>
+template <typename T, int K, int K2, int RX, int BC, int M, int F>
 __device__ __forceinline__ void split_consumer_fill(int total, Slice<T> (&W)[3][K2], const Handoff<T> &hand,
                                                     const StripGeom &geo, T *__restrict__ un,
                                                     T *__restrict__ vn, int nm, int bar_id, const Coef<T> &p) {
     constexpr int K1 = K - K2;
     constexpr int D = (M >= 1 ? (M - 1) / 2 : -1) - K1;  // computing stages, before clamping
     constexpr int ACT = D < 0 ? 0 : (D > K2 ? K2 : D);
-    split_consumer_beat<T, K, K2, RX, M % 3, ACT, (D >= 0)>(M, total, W, hand, geo, un, vn, nm, bar_id, p);
+    split_consumer_beat<T, K, K2, RX, BC, M % 3, ACT, (D >= 0)>(M, total, W, hand, geo, un, vn, nm, bar_id, p);
     if constexpr (M + 1 < F)
-        split_consumer_fill<T, K, K2, RX, M + 1, F>(total, W, hand, geo, un, vn, nm, bar_id, p);
+        split_consumer_fill<T, K, K2, RX, BC, M + 1, F>(total, W, hand, geo, un, vn, nm, bar_id, p);
 }
 
 // One work item per warp pair; `item` is the same for both warps of a pair.
@@ -221,11 +221,11 @@ __device__ __forceinline__ void temporal_split_item(int item, int bands, const T
         for (int a = 0; a < 3; ++a)
 #pragma unroll
             for (int s = 0; s < K2; ++s) zero_slice(W[a][s]);
-        split_consumer_fill<T, K, K2, RX, 0, kFill>(geo.total, W, hand, geo, un, vn, nm, bar_id, p);
+        split_consumer_fill<T, K, K2, RX, BC, 0, kFill>(geo.total, W, hand, geo, un, vn, nm, bar_id, p);
         for (int m = kFill; m <= geo.total; m += 3) {
-            split_consumer_beat<T, K, K2, RX, kFill % 3>(m, geo.total, W, hand, geo, un, vn, nm, bar_id, p);
-            split_consumer_beat<T, K, K2, RX, (kFill + 1) % 3>(m + 1, geo.total, W, hand, geo, un, vn, nm, bar_id, p);
-            split_consumer_beat<T, K, K2, RX, (kFill + 2) % 3>(m + 2, geo.total, W, hand, geo, un, vn, nm, bar_id, p);
+            split_consumer_beat<T, K, K2, RX, BC, kFill % 3>(m, geo.total, W, hand, geo, un, vn, nm, bar_id, p);
+            split_consumer_beat<T, K, K2, RX, BC, (kFill + 1) % 3>(m + 1, geo.total, W, hand, geo, un, vn, nm, bar_id, p);
+            split_consumer_beat<T, K, K2, RX, BC, (kFill + 2) % 3>(m + 2, geo.total, W, hand, geo, un, vn, nm, bar_id, p);
         }
     }
 }

@@ -150,8 +150,7 @@ int rdcnn_workspace_bytes(const rdcnn_t *h, size_t *bytes);
 /* Attach caller-owned device buffers: u and v planes (the state, updated in
  * place by rdcnn_run), scratch of at least rdcnn_workspace_bytes, and the
  * stream all later work is enqueued on.  Pointers must be device pointers;
- * 16-byte alignment enables the vectorised kernels (otherwise the generic
- * path is used).  Errors: RDCNN_EINVAL (null pointer), RDCNN_ESPACE. */
+ * 16-byte alignment enables the vectorised kernels.  Errors: RDCNN_EINVAL (null pointer), RDCNN_ESPACE. */
 int rdcnn_bind(rdcnn_t *h, void *u, void *v, void *workspace, size_t workspace_bytes,
                void *stream);
 
@@ -184,8 +183,9 @@ int rdcnn_set_state(rdcnn_t *h, const void *u0, const void *v0, int on_device);
  * read once per process, launches them plainly.  The vectorised
  * variants need NM to be a multiple of 4 (F32, BF16, F16) or 2 (F64) and
  * 16-byte (8-byte for BF16 / F16) aligned buffers;
- * AUTO falls back to GENERIC otherwise, an explicit request returns
- * RDCNN_EINVAL.  The handle's reaction and boundary apply to every
+ * otherwise an explicit request returns RDCNN_EINVAL, and AUTO runs F32
+ * planes through the temporal pipeline with elements copied one by one, others
+ * through GENERIC.  The handle's reaction and boundary apply to every
  * variant; RDCNN_VARIANT_TEMPORAL2 takes FP32 / FP64 handles only.
  * Errors: RDCNN_ESTATE, RDCNN_EINVAL, RDCNN_ECUDA. */
 int rdcnn_run(rdcnn_t *h, int64_t T, int variant, int k);
@@ -203,7 +203,8 @@ int rdcnn_run(rdcnn_t *h, int64_t T, int variant, int k);
  * out->k (0 = the handle's tuned or default depth).  Out: *variant resolved
  * from AUTO, out->k = time steps per full launch (1 for STEP1 / GENERIC),
  * out->rows = rows per warp strip (the tuned rows, else the launcher's own
- * choice; 0 for GENERIC).  Queries the current device's SM count and kernel
+ * choice; 0 for GENERIC).  Where no vectorised variant can run, AUTO is
+ * reported as GENERIC, the variant that a caller may ask for by name.  Queries the current device's SM count and kernel
  * occupancy.  Errors: RDCNN_EINVAL (as rdcnn_run would return). */
 int rdcnn_plan(const rdcnn_t *h, int *variant, rdcnn_tune *out);
 

@@ -43,7 +43,8 @@ def tune_grid(grid, x=None, trial_steps: int = 48, force: bool = False) -> dict:
         return dict(_cache[key])
     vec = 4 if grid.dtype == torch.float32 else 2
     if grid.nm % vec != 0:
-        best = {"variant": "generic", "k": 1, "rows": 0, "ms_per_step": None}
+        # no vectorised variant takes these rows: the library's own choice
+        best = {"variant": "auto", "k": 0, "rows": 0, "ms_per_step": None}
         _cache[key] = best
         return dict(best)
     cands = GRID_CANDIDATES_F64 if grid.dtype == torch.float64 else GRID_CANDIDATES_F32

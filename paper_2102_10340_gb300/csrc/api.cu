@@ -244,6 +244,9 @@ static cudaError_t launch_one(const rdcnn_t *h, int variant, int kk, const void 
     if (variant == RDCNN_VARIANT_STEP1)
         return launch_step1(h->dtype, h->reaction, h->boundary, cu, cv, nu, nv, h->nn, h->nm, h->p,
                             h->tune_rows ? h->tune_rows : default_rows_step1(h->dtype, h->nn, h->nm), s);
+    if (variant == kVariantRagged)
+        return launch_temporal_ragged(h->reaction, h->boundary, kk, cu, cv, nu, nv, h->nn, h->nm, h->p, h->tune_rows,
+                                      s);
     return launch_generic(h->dtype, h->reaction, h->boundary, cu, cv, nu, nv, h->nn, h->nm, h->p, s);
 }
 
@@ -320,8 +323,20 @@ int run_core(rdcnn_t *h, int64_t T, int variant, int k, int64_t every, MarkFn ma
     const size_t plane = (size_t)h->nn * h->nm * elem_size(h->dtype);
     char *ws = (char *)h->ws;
     void *su = ws, *sv = ws + plane_stride(plane);
+    const bool autov = (variant == RDCNN_VARIANT_AUTO);
+    const int k_arg = k;
     const int rv = resolve_variant(h, vec_ok_for(h), wide_ok_for(h), &variant, &k);
     if (rv < 0) return rv;
+    // FP32 planes that are not vector-aligned: depth does not change their
+    // bits, so AUTO steps them K at a time too (1003 x 1021, 100 steps: 758 ->
+    // 272 us).  16-bit planes round once per launch and stay with one step a
+    // launch; FP64 planes, bound by arithmetic, gain nothing from depth.  A depth that
+    // only the vectorised variants would reject is ignored here, as GENERIC
+    // ignores it.
+    if (autov && variant == RDCNN_VARIANT_GENERIC && h->dtype == RDCNN_F32) {
+        variant = kVariantRagged;
+        k = (k_arg >= 1 && k_arg <= max_k(h->dtype)) ? k_arg : h->tune_k ? h->tune_k : default_k(h->dtype, h->nn, h->nm);
+    }
     const void *cu = h->u, *cv = h->v;
     void *nu = su, *nv = sv;
     int64_t left = T;

@@ -110,9 +110,19 @@ template <> struct LaneVec<Wide<__nv_bfloat16>, 8> { typedef uint4 type; };
 template <> struct LaneVec<Wide<__half>, 8> { typedef uint4 type; };
 template <> struct LaneVec<Wide<float>, 8> { typedef Float8 type; };
 
+// A storage type E (float) of planes whose rows are not vectors:
+// NM no multiple of the lane width, or planes not 16-byte aligned.  Lanes
+// hold as many values as for E, but every element is copied and stored by
+// itself (temporal.cuh).
+template <typename E> struct Ragged { E x; };
+template <> struct LaneVec<Ragged<float>, 4> { typedef float4 type; };
+template <typename T> struct IsRagged : std::false_type {};
+template <typename E> struct IsRagged<Ragged<E>> : std::true_type {};
+
 // The element format behind a storage type (itself for the plain types).
 template <typename T> struct Base16 { typedef T type; };
 template <typename E> struct Base16<Wide<E>> { typedef E type; };
+template <typename E> struct Base16<Ragged<E>> { typedef E type; };
 
 // Lane width of the register pipelines: 4 values (2 doubles) of every
 // storage type, so that 16-bit planes share the FP32 lane layout and
@@ -126,12 +136,15 @@ template <typename E> struct Vec<Wide<E>> {
     typedef typename LaneVec<Wide<E>, 8>::type type;
 };
 
+template <typename E> struct Vec<Ragged<E>> : Vec<E> {};
+
 // Arithmetic type of a storage type: 16-bit planes are computed in FP32 and
 // rounded (to nearest, ties to even) only when stored.
 template <typename T> struct Compute { typedef T type; };
 template <> struct Compute<__nv_bfloat16> { typedef float type; };
 template <> struct Compute<__half> { typedef float type; };
 template <typename E> struct Compute<Wide<E>> { typedef float type; };
+template <typename E> struct Compute<Ragged<E>> { typedef E type; };
 template <typename T> using CT = typename Compute<T>::type;
 
 // float / double planes: arithmetic in the storage type itself.

@@ -19,6 +19,8 @@
 //              steps.  Lanes within K columns of the band edge hold stale
 //              values after K steps and do not store.
 //  k_generic   one thread per cell, scalar loads: any size and alignment.
+//              (AUTO takes it for 16-bit and FP64 planes only; FP32 planes that
+//              are not vector-aligned run k_temporal on Ragged rows.)
 //
 // All three evaluate cells with rdk::nbr_sum and rdk::cell_react, so they produce identical
 // bits for identical inputs (for 16-bit planes: at the same steps per
@@ -296,6 +298,15 @@ cudaError_t launch_temporal_wide(int dtype, int reaction, int boundary, int k, c
     });
 }
 
+// FP32 planes (the caller checks).
+cudaError_t launch_temporal_ragged(int reaction, int boundary, int k, const void *u, const void *v, void *un,
+                                   void *vn, int64_t nn, int64_t nm, const rdcnn_params &p, int rows,
+                                   cudaStream_t s) {
+    return with_depth(k, [&](auto kk) {
+        return temporal_launch<Ragged<float>, decltype(kk)::value>(reaction, boundary, u, v, un, vn, nn, nm, p, rows, s);
+    });
+}
+
 // FP32 / FP64 storage (the caller checks), every model.
 cudaError_t launch_temporal_split(int dtype, int reaction, int boundary, int k, const void *u, const void *v,
                                   void *un, void *vn, int64_t nn, int64_t nm, const rdcnn_params &p,
@@ -338,6 +349,7 @@ int plan_rows(int dtype, int reaction, int boundary, int variant, int k, int64_t
               int rows) {
     if (variant == RDCNN_VARIANT_STEP1) return rows > 0 ? rows : default_rows_step1(dtype, nn, nm);
     if (variant == RDCNN_VARIANT_GENERIC) return 0;
+    const bool ragged = (variant == kVariantRagged);
     int out = 0;
     with_dtype(dtype, [&](auto tag) {
         using T = decltype(tag);
@@ -347,6 +359,12 @@ int plan_rows(int dtype, int reaction, int boundary, int variant, int k, int64_t
                 if constexpr (K >= 2 && is_f32_f64<T>()) {
                     if (variant == RDCNN_VARIANT_TEMPORAL2) {
                         out = split_rows<T, K>(reaction, boundary, nn, nm, rows);
+                        return cudaSuccess;
+                    }
+                }
+                if constexpr (std::is_same<T, float>::value) {
+                    if (ragged) {
+                        out = temporal_rows<Ragged<float>, K>(reaction, boundary, nn, nm, rows);
                         return cudaSuccess;
                     }
                 }

@@ -43,6 +43,10 @@ constexpr int kMaxK32 = 8;  // temporal depth, FP32
 constexpr int kMaxK64 = 4;  // temporal depth, FP64
 constexpr int kMaxKWide = 4;  // temporal depth with 8 values per lane
 
+// What AUTO runs where GENERIC is the only public variant that can
+// (launch_temporal_ragged); not a value callers can pass.
+constexpr int kVariantRagged = 100;
+
 inline int vec_width(int dtype) { return dtype == RDCNN_F64 ? 2 : 4; }
 inline size_t elem_size(int dtype) {
     return dtype == RDCNN_F64 ? 8 : (dtype == RDCNN_BF16 || dtype == RDCNN_F16) ? 2 : 4;
@@ -131,6 +135,11 @@ cudaError_t launch_temporal(int dtype, int reaction, int boundary, int k, const 
 cudaError_t launch_temporal_wide(int dtype, int reaction, int boundary, int k, const void *u,
                                  const void *v, void *un, void *vn, int64_t nn, int64_t nm,
                                  const rdcnn_params &p, int rows, cudaStream_t s);
+// The temporal pipeline on rows that are not lane vectors (FP32 planes, any
+// NM and alignment).
+cudaError_t launch_temporal_ragged(int reaction, int boundary, int k, const void *u,
+                                   const void *v, void *un, void *vn, int64_t nn, int64_t nm,
+                                   const rdcnn_params &p, int rows, cudaStream_t s);
 // The temporal pipeline with the K stages split across a warp pair (k >= 2;
 // FP32 / FP64 planes, every model).
 cudaError_t launch_temporal_split(int dtype, int reaction, int boundary, int k, const void *u, const void *v,

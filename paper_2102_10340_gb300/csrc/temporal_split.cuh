@@ -52,7 +52,7 @@ __device__ __forceinline__ void hand_read(const Handoff<T> &h, int k, Slice<T> &
 template <typename T, int K1, int RX, int BC, int PH, int ACT = K1>
 __device__ __forceinline__ void split_producer_beat(int m, int total, Slice<T> (&W)[3][K1],
                                                     const RowRing<T> &ring, const Handoff<T> &hand,
-                                                    RowWalk<BC> &walk, int nn, int nm, int lc, bool rev,
+                                                    RowWalk<BC> &walk, int nn, int nm, const StripGeom &geo,
                                                     const T *__restrict__ u, const T *__restrict__ v,
                                                     int bar_id, const Coef<T> &p) {
     constexpr int V = Vec<T>::N;
@@ -60,14 +60,14 @@ __device__ __forceinline__ void split_producer_beat(int m, int total, Slice<T> (
     if (m > total) return;  // beyond the last beat: no work and no barrier (same m for both warps)
     if (m < total) {
         if (m + kRing - 1 < total) {
-            ring_issue(ring, m + kRing - 1, walk.g, nm, lc, u, v);
+            ring_issue(ring, m + kRing - 1, walk.g, nm, geo, u, v);
             walk.next(nn);
         }
         cp_async_commit();
         cp_async_wait<kRing - 1>();
         const int lane = threadIdx.x & 31;
         Slice<T> cur;
-        ring_read_bc<T, BC>(ring, m % kRing, rev, cur);
+        ring_read_bc<T, BC>(ring, m % kRing, geo.rev, cur);
 #pragma unroll
         for (int s = 0; s < K1; ++s) {
             if (s < ACT) {
@@ -142,12 +142,11 @@ __device__ __forceinline__ void split_consumer_beat(int m, int total, Slice<T> (
 template <typename T, int K1, int RX, int BC, int M, int F>
 __device__ __forceinline__ void split_producer_fill(int total, Slice<T> (&W)[3][K1], const RowRing<T> &ring,
                                                     const Handoff<T> &hand, RowWalk<BC> &walk, int nn, int nm,
-                                                    int lc, bool rev, const T *__restrict__ u,
+                                                    const StripGeom &geo, const T *__restrict__ u,
                                                     const T *__restrict__ v, int bar_id, const Coef<T> &p) {
-    split_producer_beat<T, K1, RX, BC, M % 3, (M / 2 < K1 ? M / 2 : K1)>(M, total, W, ring, hand, walk, nn, nm,
-                                                                         lc, rev, u, v, bar_id, p);
+    split_producer_beat<T, K1, RX, BC, M % 3, (M / 2 < K1 ? M / 2 : K1)>(M, total, W, ring, hand, walk, nn, nm, geo, u, v, bar_id, p);
     if constexpr (M + 1 < F)
-        split_producer_fill<T, K1, RX, BC, M + 1, F>(total, W, ring, hand, walk, nn, nm, lc, rev, u, v, bar_id, p);
+        split_producer_fill<T, K1, RX, BC, M + 1, F>(total, W, ring, hand, walk, nn, nm, geo, u, v, bar_id, p);
 }
 
 // Fill beats 0 .. F-1 of the consumer (equivalent beat M - 1): local stage j
@@ -199,20 +198,18 @@ __device__ __forceinline__ void temporal_split_item(int item, int bands, const T
 #pragma unroll
         for (int j = 0; j < kRing - 1; ++j) {
             if (j < geo.total) {
-                ring_issue(ring, j, walk.g, nm, geo.lc, u, v);
+                ring_issue(ring, j, walk.g, nm, geo, u, v);
                 walk.next(nn);
             }
             cp_async_commit();
         }
-        split_producer_fill<T, K1, RX, BC, 0, kFill>(geo.total, W, ring, hand, walk, nn, nm, geo.lc, geo.rev, u, v,
+        split_producer_fill<T, K1, RX, BC, 0, kFill>(geo.total, W, ring, hand, walk, nn, nm, geo, u, v,
                                                      bar_id, p);
         for (int m = kFill; m <= geo.total; m += 3) {
-            split_producer_beat<T, K1, RX, BC, kFill % 3>(m, geo.total, W, ring, hand, walk, nn, nm, geo.lc, geo.rev,
+            split_producer_beat<T, K1, RX, BC, kFill % 3>(m, geo.total, W, ring, hand, walk, nn, nm, geo,
                                                           u, v, bar_id, p);
-            split_producer_beat<T, K1, RX, BC, (kFill + 1) % 3>(m + 1, geo.total, W, ring, hand, walk, nn, nm, geo.lc,
-                                                                geo.rev, u, v, bar_id, p);
-            split_producer_beat<T, K1, RX, BC, (kFill + 2) % 3>(m + 2, geo.total, W, ring, hand, walk, nn, nm, geo.lc,
-                                                                geo.rev, u, v, bar_id, p);
+            split_producer_beat<T, K1, RX, BC, (kFill + 1) % 3>(m + 1, geo.total, W, ring, hand, walk, nn, nm, geo, u, v, bar_id, p);
+            split_producer_beat<T, K1, RX, BC, (kFill + 2) % 3>(m + 2, geo.total, W, ring, hand, walk, nn, nm, geo, u, v, bar_id, p);
         }
         cp_async_wait<0>();
     } else {

@@ -98,7 +98,7 @@ enum { RDCNN_F32 = 0, RDCNN_F64 = 1,
 enum { RDCNN_REACTION_FHN = 0,                    /* Eq. 2-3 */
        RDCNN_REACTION_NONE = 1,                   /* f1 = f2 = 0: pure diffusion (testing) */
        RDCNN_REACTION_CENN = 2 };                 /* Chua-Yang cell (see above) */
-enum { RDCNN_VARIANT_AUTO = 0,                    /* library's choice (temporal when possible) */
+enum { RDCNN_VARIANT_AUTO = 0,                    /* library's choice */
        RDCNN_VARIANT_STEP1 = 1,                   /* one launch per time step, float4/double2 rows */
        RDCNN_VARIANT_TEMPORAL = 2,                /* k time steps fused per launch */
        RDCNN_VARIANT_GENERIC = 3,                 /* scalar path: any size, any alignment */
@@ -185,7 +185,8 @@ int rdcnn_set_state(rdcnn_t *h, const void *u0, const void *v0, int on_device);
  * 16-byte (8-byte for BF16 / F16) aligned buffers;
  * otherwise an explicit request returns RDCNN_EINVAL, and AUTO runs F32
  * planes through the temporal pipeline with elements copied one by one, others
- * through GENERIC.  The handle's reaction and boundary apply to every
+ * through GENERIC.  AUTO on F64 planes is STEP1 unless a depth is asked for
+ * (k or tune->k).  The handle's reaction and boundary apply to every
  * variant; RDCNN_VARIANT_TEMPORAL2 takes FP32 / FP64 handles only.
  * Errors: RDCNN_ESTATE, RDCNN_EINVAL, RDCNN_ECUDA. */
 int rdcnn_run(rdcnn_t *h, int64_t T, int variant, int k);

@@ -198,8 +198,8 @@ bool adj_streams(rdcnn_t *h) {
 // launches of a stretch alternate between the scratch pair and the stretch's
 // destination and end in the destination, so no launch reads the planes it
 // writes.
-// Launch shapes: the temporal kernel at the size's default depth between
-// checkpoints; for a full tape (S = 1) the store-all pipeline, which writes
+// Launch shapes: what AUTO runs (the temporal kernel at the size's default
+// depth; FP64 the single step) between checkpoints; for a full tape (S = 1) the store-all pipeline, which writes
 // ka consecutive states per launch.  Every variant computes the same bits,
 // so the states are those rdcnn_run produces.
 template <typename T>
@@ -220,7 +220,7 @@ int record_states(int dtype, int reaction, int boundary, int64_t nn, int64_t nm,
             q += kk;
         }
     }
-    const int kf = default_k(dtype, nn, nm);
+    const int kf = auto_single_step(dtype) ? 1 : default_k(dtype, nn, nm);
     auto advance = [&](const void *cu, const void *cv, int64_t len, void *ou, void *ov) -> cudaError_t {
         const int64_t nl = (len + kf - 1) / kf;
         for (int64_t j = 0; j < nl; ++j) {
@@ -228,7 +228,11 @@ int record_states(int dtype, int reaction, int boundary, int64_t nn, int64_t nm,
             const bool to_dest = ((nl - 1 - j) % 2) == 0;
             void *nu = to_dest ? ou : tu;
             void *nv = to_dest ? ov : tv;
-            const cudaError_t le = launch_temporal(dtype, reaction, boundary, kk, cu, cv, nu, nv, nn, nm, p, 0, s);
+            const cudaError_t le =
+                auto_single_step(dtype)
+                    ? launch_step1(dtype, reaction, boundary, cu, cv, nu, nv, nn, nm, p,
+                                   default_rows_step1(dtype, nn, nm), s)
+                    : launch_temporal(dtype, reaction, boundary, kk, cu, cv, nu, nv, nn, nm, p, 0, s);
             if (le != cudaSuccess) return le;
             cu = nu; cv = nv;
         }

@@ -198,7 +198,11 @@ static int resolve_variant(const rdcnn_t *h, bool vec_ok, bool wide_ok, int *var
         if (*k < 1 || *k > kMaxKWide) return set_error(RDCNN_EINVAL, "k must be in 1..%d for the wide variant", kMaxKWide);
         return RDCNN_OK;
     }
-    if (*variant == RDCNN_VARIANT_AUTO) *variant = vec_ok ? RDCNN_VARIANT_TEMPORAL : RDCNN_VARIANT_GENERIC;
+    if (*variant == RDCNN_VARIANT_AUTO) {
+        *variant = !vec_ok ? RDCNN_VARIANT_GENERIC
+                   : auto_single_step(h->dtype) && *k == 0 && h->tune_k == 0 ? RDCNN_VARIANT_STEP1  // no depth asked for
+                                                                             : RDCNN_VARIANT_TEMPORAL;
+    }
     if ((*variant == RDCNN_VARIANT_STEP1 || *variant == RDCNN_VARIANT_TEMPORAL ||
          *variant == RDCNN_VARIANT_TEMPORAL2) && !vec_ok)
         return set_error(RDCNN_EINVAL,
@@ -330,7 +334,7 @@ int run_core(rdcnn_t *h, int64_t T, int variant, int k, int64_t every, MarkFn ma
     // FP32 planes that are not vector-aligned: depth does not change their
     // bits, so AUTO steps them K at a time too (1003 x 1021, 100 steps: 758 ->
     // 272 us).  16-bit planes round once per launch and stay with one step a
-    // launch; FP64 planes, bound by arithmetic, gain nothing from depth.  A depth that
+    // launch; FP64 planes are fastest with one (auto_single_step).  A depth that
     // only the vectorised variants would reject is ignored here, as GENERIC
     // ignores it.
     if (autov && variant == RDCNN_VARIANT_GENERIC && h->dtype == RDCNN_F32) {

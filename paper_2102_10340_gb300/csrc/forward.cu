@@ -386,24 +386,34 @@ int plan_rows(int dtype, int reaction, int boundary, int variant, int k, int64_t
 // square grids): 128^2-256^2 k=4, 512^2 k=6, 1024^2 k=4, >= 2048^2 k=8.
 // Small grids are latency/launch bound, where fewer, shallower stages in
 // more warps win; large grids are FP32-pipe bound, where depth amortises
-// the halo.  FP64 is capped at its maximum depth.
+// the halo.  FP64: 2, see auto_single_step.
 int default_k(int dtype, int64_t nn, int64_t nm) {
     const int64_t cells = nn * nm;
-    int k;
-    if (cells >= (int64_t(1) << 21)) k = 8;
-    else if (cells >= (int64_t(1) << 19)) k = 4;
-    else if (cells >= (int64_t(1) << 17)) k = 6;
-    else k = 4;
-    return std::min(k, max_k(dtype));
+    if (dtype == RDCNN_F64) return 2;
+    if (cells >= (int64_t(1) << 21)) return 8;
+    if (cells >= (int64_t(1) << 19)) return 4;
+    if (cells >= (int64_t(1) << 17)) return 6;
+    return 4;
 }
+
+// FP64 runs at 1/64 of the FP32 rate, so the FP64 pipe bounds every grid that
+// fills the GPU, and a halo cell costs as much as an owned one: the single
+// step, which computes no cell twice, beats every depth at every size.  us a
+// step (k = 4 / best depth / single step): 64^2 6.5 / 3.6 / 2.3, 256^2 6.5 /
+// 4.7 / 3.6, 512^2 16.6 / 9.8 / 9.1, 1024^2 37.1 / 33.0 / 29.6, 2048^2 135 /
+// 121 / 110.
+bool auto_single_step(int dtype) { return dtype == RDCNN_F64; }
 
 // The single-step kernel is fastest with short strips (more warps in flight);
 // the 16-bit single step (the ring pipeline at depth 1, 8 values per lane)
 // with 32-row strips (measured at 4096^2, bf16: 4 / 8 / 16 / 32 / 64 rows =
 // 507 / 570 / 627 / 672 / 574 Gcell/s).
+// FP64: one row while that leaves warp slots free, else two (us a step, 1 / 2 /
+// 4 / 8 rows: 64^2 2.3 / 3.6 / 5.6 / 10.2, 256^2 3.6 / 3.7 / 5.9 / 10.5, 512^2
+// 10.4 / 9.1 / 10.0 / 11.1, 2048^2 120 / 110 / 110 / 114).
 int default_rows_step1(int dtype, int64_t nn, int64_t nm) {
-    (void)nn; (void)nm;
-    return is_16bit(dtype) ? 32 : dtype == RDCNN_F32 ? 2 : 4;
+    if (dtype == RDCNN_F64) return nn * nm <= (int64_t(1) << 16) ? 1 : 2;
+    return is_16bit(dtype) ? 32 : 2;
 }
 
 }  // namespace rdk

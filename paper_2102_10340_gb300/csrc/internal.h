@@ -173,5 +173,7 @@ cudaError_t launch_init(int dtype, const void *x, void *u, void *v, double ka, i
 // itself when given rows <= 0.
 int default_rows_step1(int dtype, int64_t nn, int64_t nm);
 int default_k(int dtype, int64_t nn, int64_t nm);
+// Whether AUTO takes the single-step kernel rather than a temporal depth.
+bool auto_single_step(int dtype);
 
 }  // namespace rdk

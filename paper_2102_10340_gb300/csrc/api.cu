@@ -317,6 +317,9 @@ static bool ensure_graph(rdcnn_t *h, int variant, int k, void *su, void *sv) {
     return true;
 }
 
+// Most steps of one resident launch: 1 .. 7 ms.
+constexpr int64_t kResidentSteps = 8192;
+
 int run_core(rdcnn_t *h, int64_t T, int variant, int k, int64_t every, MarkFn mark, void *ctx) {
     if (!h) return set_error(RDCNN_EINVAL, "handle is NULL");
     if (!h->bound) return set_error(RDCNN_ESTATE, "handle is not bound");
@@ -344,8 +347,26 @@ int run_core(rdcnn_t *h, int64_t T, int variant, int k, int64_t every, MarkFn ma
     const void *cu = h->u, *cv = h->v;
     void *nu = su, *nv = sv;
     int64_t left = T;
+    // small FP32 grids with no depth or strip length asked for: whole stretches of
+    // the run in one launch, in place
+    if (autov && k_arg == 0 && h->tune_k == 0 && h->tune_rows == 0 && h->dtype == RDCNN_F32 &&
+        resident_fits(h->nn, h->nm)) {
+        while (left > 0) {
+            int64_t n = std::min<int64_t>(left, kResidentSteps);
+            if (every > 0) n = std::min<int64_t>(n, every - (T - left) % every);
+            const cudaError_t e = launch_resident(h->reaction, h->boundary, h->u, h->v, h->nn, h->nm, h->p, n, h->stream);
+            if (e == cudaErrorNotSupported) break;  // no room for the cluster: the launches below
+            if (e != cudaSuccess) return cuda_error(e, "resident kernel launch");
+            left -= n;
+            if (every > 0 && (T - left) % every == 0 && mark) {
+                const int rc = mark(ctx, T - left, h->u, h->v);
+                if (rc < 0) return rc;
+            }
+        }
+        if (left == 0) return RDCNN_OK;
+    }
     // launch-bound runs: replay whole groups of full-depth launches as a graph
-    const int64_t full = T / k;
+    const int64_t full = left / k;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (every == 0 && !mark && full >= 2 * kGraphLaunches && h->nn * h->nm * (int64_t)k <= (int64_t(1) << 23) &&
         cudaStreamIsCapturing(h->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&

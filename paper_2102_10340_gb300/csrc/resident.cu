@@ -1,0 +1,65 @@
+// resident.cu -- which runs the cluster-resident kernel (resident.cuh) takes,
+// and in which shape.
+#include <algorithm>
+
+#include "resident_launch.cuh"
+
+extern template RDK_RESIDENT_SIG(2);
+extern template RDK_RESIDENT_SIG(4);
+extern template RDK_RESIDENT_SIG(8);
+
+namespace rdk {
+
+namespace {
+
+// Lane width, blocks of the cluster and warps of a block; every warp has
+// 1 .. kResRows rows.  V = 0: the grid does not fit.
+struct ResShape {
+    int V = 0, blocks = 0, warps = 0;
+};
+
+// Sixteen blocks whatever the size (us a step with 16 / 8 / 4 / 1 blocks: 64^2
+// 0.25 / 0.25 / 0.32 / 0.57, 128^2 0.32 / 0.41 / 0.60 / -, 256^2 0.62 / 0.92 / - / -,
+// with plain rows handed on), and as many rows a warp as leave one warp to each
+// of an SM's four schedulers, at most four: 64^2 with 1 / 2 / 4 rows 0.20 / 0.22 /
+// 0.26, 256^2 with 2 / 4 rows 0.52 / 0.49, 512 x 256 with 4 rows 0.75.
+// Against the launches it stands for (k = 4 or 6, replayed as a graph) it is
+// faster over all of its range and at any number of steps (T = 1024, us: 16 x 256
+// 805 -> 345, 64^2 857 -> 181, 1024 x 128 1187 -> 740, 512 x 256 1187 -> 763,
+// 251 x 253 1412 -> 709; T = 2: one launch in the place of one and two copies).
+ResShape resident_shape(int64_t nn, int64_t nm) {
+    ResShape s;
+    if (nm < 16 || nm > 256 || nn < 1) return s;
+    const int V = nm <= 64 ? 2 : nm <= 128 ? 4 : 8;
+    const int most = V == 8 ? ResWarps<8>::value : ResWarps<4>::value;
+    const int blocks = (int)std::min<int64_t>(16, nn);
+    const int64_t per_block = (nn + blocks - 1) / blocks;
+    const int64_t rows = std::min<int64_t>(kResRows, (per_block + 3) / 4);
+    // no more warps than rows
+    const int64_t warps = std::min<int64_t>((per_block + rows - 1) / rows, nn / blocks);
+    if (warps > most || (nn + blocks * warps - 1) / (blocks * warps) > kResRows) return s;
+    s.V = V;
+    s.blocks = blocks;
+    s.warps = (int)warps;
+    return s;
+}
+
+}  // namespace
+
+bool resident_fits(int64_t nn, int64_t nm) { return resident_shape(nn, nm).V != 0; }
+
+cudaError_t launch_resident(int reaction, int boundary, void *u, void *v, int64_t nn, int64_t nm,
+                            const rdcnn_params &p, int64_t steps, cudaStream_t s) {
+    const ResShape q = resident_shape(nn, nm);
+    auto go = [&](auto vv) {
+        return resident_launch_v<decltype(vv)::value>(reaction, boundary, u, v, nn, nm, p, q.blocks, q.warps, steps, s);
+    };
+    switch (q.V) {
+        case 2: return go(IntC<2>{});
+        case 4: return go(IntC<4>{});
+        case 8: return go(IntC<8>{});
+        default: return cudaErrorNotSupported;
+    }
+}
+
+}  // namespace rdk

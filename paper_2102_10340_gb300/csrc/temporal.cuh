@@ -202,7 +202,8 @@ template <int BC> struct RowWalk {
 // pair sums acc(j) = row_{q-1}(j+1) + row_q(j) instead of rows q - 1 and q:
 // the sum of a cell is its own new pair (row_q(j+1) + C(j)) plus the old pair
 // one column to the west -- two additions per field instead of three, at the
-// same registers and the same two shuffles.  4096^2, K = 8: @PAIR@
+// same registers and the same two shuffles.  4096^2, K = 8:
+// 92.7 -> 82.7 us a launch.
 // Zero flux: rows q - 1 and q, three additions (nbr_sum says why).
 // CeNN cell (OUT): the sums run over the outputs y = clamp(x), clamped once
 // when a row arrives and kept (pair sums and y of row q on the torus, y of

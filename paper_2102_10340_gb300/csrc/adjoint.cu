@@ -32,7 +32,8 @@
 // steps).  Segments are then processed last to first: k_forward_all rebuilds
 // the segment's states K per launch (every stage of the temporal pipeline is
 // stored), and k_adjoint_pipe walks them backwards K steps per launch with
-// the same register pipeline running the co-state update.  With more than
+// the same register pipeline running the co-state update (FP64 with no depth
+// asked for: single steps both ways, k_step1 and k_adjoint_step).  With more than
 // one segment the rebuilds run on a second stream into two alternating
 // buffer sets, so the rebuild of segment s - 1 overlaps the reverse sweep of
 // segment s (events order each rebuild after the reverse sweep that last read
@@ -57,22 +58,127 @@ RDK_EXTERN_ADJ(double, 1, 2) RDK_EXTERN_ADJ(double, 2, 2) RDK_EXTERN_ADJ(double,
 namespace rdk {
 
 namespace {
-// Sum per-warp partials (fixed order), scale by dt: out[q] = dt * sum_w partial[w][q].
+// Sum the partial records (fixed order), one block per gene entry, scale by dt:
+// out[q] = dt * sum_w partial[w][q].
 __global__ void __launch_bounds__(256)
-k_reduce_partials(const double *__restrict__ partial, int nwarps, double dt, double *__restrict__ out) {
+k_reduce_partials(const double *__restrict__ partial, int n, double dt, double *__restrict__ out) {
     __shared__ double sh[256];
-    for (int q = 0; q < 6; ++q) {
-        double s = 0.0;
-        for (int w = threadIdx.x; w < nwarps; w += 256) s += partial[(int64_t)w * 6 + q];
-        sh[threadIdx.x] = s;
-        __syncthreads();
-        for (int h = 128; h > 0; h >>= 1) {
-            if ((int)threadIdx.x < h) sh[threadIdx.x] += sh[threadIdx.x + h];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) out[q] = dt * sh[0];
+    const int q = blockIdx.x;
+    double s = 0.0;
+    for (int w = threadIdx.x; w < n; w += 256) s += partial[(int64_t)w * 6 + q];
+    sh[threadIdx.x] = s;
+    __syncthreads();
+    for (int h = 128; h > 0; h >>= 1) {
+        if ((int)threadIdx.x < h) sh[threadIdx.x] += sh[threadIdx.x + h];
         __syncthreads();
     }
+    if (threadIdx.x == 0) out[q] = dt * sh[0];
+}
+
+// One reverse step of FP64 planes, a warp per 64 columns and `rows` rows.  The
+// FP64 pipe (1/64 of the FP32 rate) bounds this step once the grid fills the
+// GPU, so it computes no cell twice, unlike the pipeline (k_adjoint_pipe), and
+// its warps are short: on a small grid the pipeline's few strips leave most SMs
+// idle.  us a step of the reverse sweep, pipeline with k = 2 / this: 64^2 11.1 /
+// 5.8, 128^2 11.2 / 6.4, 256^2 16.9 / 9.8, 512^2 31.7 / 24.7, 1024^2 101 / 78.
+// Sums: each lane's six, added over groups of four lanes and then to the
+// group's record in `partial` (one record per 4 lanes of every warp, read and
+// written by the same lane at each launch), so no launch reduces a whole warp.
+constexpr int kRevBlock = 64;
+constexpr int kRevRecords = 8;  // records per warp
+
+template <int RX, int BC>
+__global__ void __launch_bounds__(kRevBlock)
+k_adjoint_step(const double *__restrict__ lu, const double *__restrict__ lv, double *__restrict__ lun,
+               double *__restrict__ lvn, const double *__restrict__ u, const double *__restrict__ v,
+               double *__restrict__ partial, int nn, int nm, int bands, int nwarps, int rows, AdjCoef<double> p) {
+    constexpr int V = 2;
+    constexpr bool zf = (BC == BC_MIRROR);
+    pdl_wait();
+    const int lane = threadIdx.x & 31;
+    const int wid = blockIdx.x * (kRevBlock / 32) + (threadIdx.x >> 5);
+    if (wid >= nwarps) return;  // whole warps only
+    const int col = (wid % bands) * 32 * V + lane * V;
+    const bool active = col < nm;
+    const int colw = (col == 0) ? (zf ? 0 : nm - 1) : col - 1;
+    const int cole = (col + V >= nm) ? (zf ? nm - 1 : 0) : col + V;
+    const bool edge_w = (lane == 0);
+    const bool edge_e = active && (lane == 31 || col + V >= nm);
+    const int r0 = wid / bands * rows, r1 = min(r0 + rows, nn);
+    double rg[6] = {0, 0, 0, 0, 0, 0};
+    for (int r = r0; r < r1; ++r) {
+        const int64_t rn = r == 0 ? (zf ? 0 : nn - 1) : r - 1, rs = r + 1 == nn ? (zf ? r : 0) : r + 1;
+        const int64_t at = (int64_t)r * nm + col;
+        Slice<double> n, c, s, st;
+        zero_slice(n); zero_slice(c); zero_slice(s); zero_slice(st);
+        double ewu = 0, ewv = 0, eeu = 0, eev = 0;
+        if (active) {
+            load_slice(n, lu, lv, rn * nm + col);
+            load_slice(c, lu, lv, at);
+            load_slice(s, lu, lv, rs * nm + col);
+            load_slice(st, u, v, at);
+        }
+        if (edge_w) { ewu = __ldg(lu + (int64_t)r * nm + colw); ewv = __ldg(lv + (int64_t)r * nm + colw); }
+        if (edge_e) { eeu = __ldg(lu + (int64_t)r * nm + cole); eev = __ldg(lv + (int64_t)r * nm + cole); }
+        double wu = __shfl_up_sync(kFull, c.u[V - 1], 1), eu = __shfl_down_sync(kFull, c.u[0], 1);
+        double wv = __shfl_up_sync(kFull, c.v[V - 1], 1), ev = __shfl_down_sync(kFull, c.v[0], 1);
+        if (edge_w) { wu = ewu; wv = ewv; }
+        if (edge_e) { eu = eeu; ev = eev; }
+        Slice<double> out;
+#pragma unroll
+        for (int e = 0; e < V; ++e)
+            reverse_cell<double, RX>(c.u[e], c.v[e], nbr_sum<BC>(n.u[e], s.u[e], e == 0 ? wu : c.u[0], e == 0 ? c.u[1] : eu),
+                                     nbr_sum<BC>(n.v[e], s.v[e], e == 0 ? wv : c.v[0], e == 0 ? c.v[1] : ev), st.u[e],
+                                     st.v[e], p, active, rg, out.u[e], out.v[e]);
+        if (active) {
+            store_vec<double>(lun + at, out.u);
+            store_vec<double>(lvn + at, out.v);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+        rg[q] = add_rn(rg[q], __shfl_xor_sync(kFull, rg[q], 1));
+        rg[q] = add_rn(rg[q], __shfl_xor_sync(kFull, rg[q], 2));
+    }
+    if ((lane & 3) == 0) {
+        double *rec = partial + ((int64_t)wid * kRevRecords + lane / 4) * 6;
+#pragma unroll
+        for (int q = 0; q < 6; ++q) rec[q] = add_rn(rec[q], rg[q]);
+    }
+    pdl_trigger();
+}
+
+struct StepShape {
+    int bands, nwarps, rows;
+    size_t bytes;  // of the records
+};
+
+// Rows per warp: one up to 2^18 cells, four above, where the sums' additions (18
+// of 68 FP64 instructions of a one-row warp) weigh more.  us a step of the whole
+// reverse sweep, rebuilds included, with 1 / 2 / 4 / 8 rows: 128^2 6.4 / 8.1 / 11.4
+// / 18.8, 512^2 24.7 / 24.9 / 27.8 / 31.9, 1024^2 91.6 / 82.8 / 77.8 / 78.8.
+StepShape step_shape(int64_t nn, int64_t nm) {
+    StepShape q;
+    q.rows = nn * nm <= (int64_t(1) << 18) ? 1 : 4;
+    q.bands = (int)((nm + 63) / 64);
+    q.nwarps = q.bands * (int)((nn + q.rows - 1) / q.rows);
+    q.bytes = (size_t)q.nwarps * kRevRecords * 6 * sizeof(double);
+    return q;
+}
+
+cudaError_t reverse_step(int reaction, int boundary, const void *lu, const void *lv, void *lun, void *lvn, const void *u,
+                         const void *v, double *partial, int64_t nn, int64_t nm, const StepShape &q,
+                         const rdcnn_params &p, cudaStream_t s) {
+    const AdjCoef<double> c = make_adj_coef<double>(p, reaction);
+    const unsigned grid = (unsigned)((q.nwarps + kRevBlock / 32 - 1) / (kRevBlock / 32));
+    return with_model(reaction, boundary, [&](auto rx, auto bc) {
+        const cudaError_t e = launch_k(k_adjoint_step<decltype(rx)::value, decltype(bc)::value>, grid, kRevBlock, 0, s,
+                                       (const double *)lu, (const double *)lv, (double *)lun, (double *)lvn,
+                                       (const double *)u, (const double *)v, partial, (int)nn, (int)nm, q.bands,
+                                       q.nwarps, q.rows, c);
+        count_launches(1);
+        return e;
+    });
 }
 
 // Depth of the recompute / reverse launches (handle tune k, else these), and
@@ -223,8 +329,10 @@ int record_states(int dtype, int reaction, int boundary, int64_t nn, int64_t nm,
     const int kf = auto_single_step(dtype) ? 1 : default_k(dtype, nn, nm);
     auto advance = [&](const void *cu, const void *cv, int64_t len, void *ou, void *ov) -> cudaError_t {
         const int64_t nl = (len + kf - 1) / kf;
+        int64_t t = 0;
         for (int64_t j = 0; j < nl; ++j) {
-            const int kk = (int)std::min<int64_t>(kf, len - j * kf);
+            const int kk = (int)((len - t + nl - j - 1) / (nl - j));  // even depths (the bits do not depend on them)
+            t += kk;
             const bool to_dest = ((nl - 1 - j) % 2) == 0;
             void *nu = to_dest ? ou : tu;
             void *nv = to_dest ? ov : tv;
@@ -276,10 +384,17 @@ int reverse_sweep(rdcnn_t *h, int64_t nn, int64_t nm, const rdcnn_params &p, int
     double *gout = (double *)(ws + L.out_off);
     const PipeShape sh = pipe_shape(dtype, nn, nm, L.H);
     const int ka = L.ka;  // depth of recompute / reverse launches
+    // FP64 with no depth asked for goes step by step (k_adjoint_step); the records
+    // of its sums are more than the layout's, and lie in segment slot 0 of set 0,
+    // which holds no state (step 0 of a segment is its checkpoint).
+    const StepShape one = step_shape(nn, nm);
+    const bool single = std::is_same<T, double>::value && h->tune_k == 0 && !L.full && one.bytes <= 2 * L.plane;
+    if (single) partial = (double *)(ws + L.seg_off);
+    const size_t partial_bytes = single ? one.bytes : (size_t)sh.nwarps * 6 * sizeof(double);
 
     cudaError_t e = cudaMemcpyAsync(lam_u[0], dLdu_T, bytes, cudaMemcpyDeviceToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(lam_v[0], dLdv_T, bytes, cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(partial, 0, (size_t)sh.nwarps * 6 * sizeof(double), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(partial, 0, partial_bytes, s);
     if (e != cudaSuccess) return cuda_error(e, "adjoint setup copies");
     if (overlap) {  // the rebuilds read the checkpoints
         e = cudaEventRecord(h->adj_ev[0], s);
@@ -289,6 +404,14 @@ int reverse_sweep(rdcnn_t *h, int64_t nn, int64_t nm, const rdcnn_params &p, int
     int cur = 0;
     auto sweep_back = [&](int64_t len, auto state_u, auto state_v) -> cudaError_t {
         for (int64_t qh = len; qh > 0;) {
+            if (single) {
+                const cudaError_t le = reverse_step(reaction, boundary, lam_u[cur], lam_v[cur], lam_u[cur ^ 1], lam_v[cur ^ 1],
+                                                    state_u(qh - 1), state_v(qh - 1), partial, nn, nm, one, p, s);
+                if (le != cudaSuccess) return le;
+                cur ^= 1;
+                --qh;
+                continue;
+            }
             const int kk = (int)std::min<int64_t>(ka, qh);
             StagePlanes<T> st{};
             for (int j = 0; j < kk; ++j) { st.u[j] = state_u(qh - 1 - j); st.v[j] = state_v(qh - 1 - j); }
@@ -316,6 +439,13 @@ int reverse_sweep(rdcnn_t *h, int64_t nn, int64_t nm, const rdcnn_params &p, int
             if (e != cudaSuccess) return fail(e, "adjoint stream order");
         }
         for (int64_t q = 0; q + 1 < len;) {
+            if (single) {
+                e = launch_step1(dtype, reaction, boundary, state_u(q), state_v(q), seg_u(q + 1), seg_v(q + 1), nn, nm, p,
+                                 default_rows_step1(dtype, nn, nm), rs);
+                if (e != cudaSuccess) return fail(e, "adjoint recompute");
+                ++q;
+                continue;
+            }
             const int kk = (int)std::min<int64_t>(ka, len - 1 - q);
             StagePlanes<T> pl{};
             for (int j = 0; j < kk; ++j) { pl.u[j] = seg_u(q + 1 + j); pl.v[j] = seg_v(q + 1 + j); }
@@ -335,7 +465,7 @@ int reverse_sweep(rdcnn_t *h, int64_t nn, int64_t nm, const rdcnn_params &p, int
             if (e != cudaSuccess) return fail(e, "adjoint stream order");
         }
     }
-    k_reduce_partials<<<1, 256, 0, s>>>(partial, sh.nwarps, p.dt, gout);
+    k_reduce_partials<<<6, 256, 0, s>>>(partial, single ? one.nwarps * kRevRecords : sh.nwarps, p.dt, gout);
     count_launches(1);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_error(e, "gradient reduction");
@@ -345,6 +475,11 @@ int reverse_sweep(rdcnn_t *h, int64_t nn, int64_t nm, const rdcnn_params &p, int
     if (e == cudaSuccess) e = cudaMemcpyAsync(hg, gout, sizeof(hg), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_error(e, "adjoint results");
+    if (single && reaction == RDCNN_REACTION_FHN) {  // as ReversePolicy::flush scales its sums
+        hg[4] = -(hg[4] + p.a * hg[2]);
+        hg[3] *= p.eps;
+        hg[2] *= -p.eps;
+    }
     for (int q = 0; q < 6; ++q) grad[q] = hg[q];
     return RDCNN_OK;
 }

@@ -49,6 +49,50 @@ __device__ __forceinline__ T warp_sum_t(T x) {
     return x;
 }
 
+// One cell of a reverse step: co-state (luc, lvc) with neighbour sums su, sv and
+// the state (uc, vc) before the step -> the co-state before it; `own` cells add
+// to the six gene sums rg: u Lap(lu), v Lap(lv), lv, lv v, lv (u - b v), lu u.
+// With the centre term folded in, like the forward:
+//   lu + dt [ Du s(lu) + (c - 4 Du - u^2) lu - eps lv ]
+//   lv + dt [ Dv s(lv) + (eps b - 4 Dv) lv - lu ]
+template <typename T, int RX>
+__device__ __forceinline__ void reverse_cell(T luc, T lvc, T su, T sv, T uc, T vc, const AdjCoef<T> &p, bool own,
+                                             T (&rg)[6], T &out_u, T &out_v) {
+    if constexpr (RX == RX_CENN) {
+        // -lu + y'(u) (c lu + Du sum_nbr lu); y' in {0, 1}, so the product is exact
+        const T slope = fabs(uc) < T(1) ? T(1) : T(0);
+        const T back = fma_rn(p.Du, su, mul_rn(p.cm4, luc));
+        out_u = fma_rn(p.dt, fma_rn(slope, back, -luc), luc);
+        out_v = fma_rn(p.dt, luc, lvc);
+        if (own) {
+            const T yc = clamp1(uc);
+            rg[0] = fma_rn(yc, su, rg[0]);   // y(u) sum_nbr lu  (Du)
+            rg[5] = fma_rn(luc, yc, rg[5]);  // lu y(u)          (c)
+        }
+        return;
+    }
+    T ru, rv;
+    if (RX == RX_FHN) {
+        ru = fma_rn(fma_rn(-uc, uc, p.cm4), luc, mul_rn(p.meps, lvc));
+        rv = fma_rn(p.ebm4, lvc, -luc);
+    } else {
+        ru = mul_rn(p.cm4, luc);
+        rv = mul_rn(p.ebm4, lvc);
+    }
+    out_u = fma_rn(p.dt, fma_rn(p.Du, su, ru), luc);
+    out_v = fma_rn(p.dt, fma_rn(p.Dv, sv, rv), lvc);
+    if (own) {
+        rg[0] = fma_rn(uc, fma_rn(T(-4), luc, su), rg[0]);     // u Lap(lu)
+        rg[1] = fma_rn(vc, fma_rn(T(-4), lvc, sv), rg[1]);     // v Lap(lv)
+        if (RX == RX_FHN) {
+            rg[2] = add_rn(rg[2], lvc);                        // lv        (x -eps)
+            rg[3] = fma_rn(lvc, vc, rg[3]);                    // lv v      (x eps)
+            rg[4] = fma_rn(lvc, fma_rn(p.mb, vc, uc), rg[4]);  // lv (u - b v)
+            rg[5] = fma_rn(luc, uc, rg[5]);                    // lu u
+        }
+    }
+}
+
 // Reverse policy for the K-stage pipeline.  The pipeline streams the
 // co-state (Slice.u = lu, Slice.v = lv, time t_hi first); stage s produces
 // the co-state at time t_hi - s - 1 from the one at t_hi - s, using the state
@@ -103,48 +147,10 @@ struct ReversePolicy {
         const T *stv = reinterpret_cast<const T *>(&sv4);
 #pragma unroll
         for (int e = 0; e < V; ++e) {
-            const T luc = B.u[e], lvc = B.v[e];
-            const T su = nu[e], sv = nv[e];
             // a mirrored lane holds its state vector reversed, like its co-state
             const bool flip = (BC == BC_MIRROR) && geo.rev;
-            const T uc = flip ? stu[V - 1 - e] : stu[e];
-            const T vc = flip ? stv[V - 1 - e] : stv[e];
-            // co-state update with the centre term folded in, like the forward:
-            //   lu + dt [ Du s(lu) + (c - 4 Du - u^2) lu - eps lv ]
-            //   lv + dt [ Dv s(lv) + (eps b - 4 Dv) lv - lu ]
-            if constexpr (RX == RX_CENN) {
-                // -lu + y'(u) (c lu + Du sum_nbr lu); y' in {0, 1}, so the product is exact
-                const T slope = fabs(uc) < T(1) ? T(1) : T(0);
-                const T back = fma_rn(p.Du, su, mul_rn(p.cm4, luc));
-                out.u[e] = fma_rn(p.dt, fma_rn(slope, back, -luc), luc);
-                out.v[e] = fma_rn(p.dt, luc, lvc);
-                if (own) {
-                    const T yc = clamp1(uc);
-                    rg[0] = fma_rn(yc, su, rg[0]);   // y(u) sum_nbr lu  (Du)
-                    rg[5] = fma_rn(luc, yc, rg[5]);  // lu y(u)          (c)
-                }
-                continue;
-            }
-            T ru, rv;
-            if (RX == RX_FHN) {
-                ru = fma_rn(fma_rn(-uc, uc, p.cm4), luc, mul_rn(p.meps, lvc));
-                rv = fma_rn(p.ebm4, lvc, -luc);
-            } else {
-                ru = mul_rn(p.cm4, luc);
-                rv = mul_rn(p.ebm4, lvc);
-            }
-            out.u[e] = fma_rn(p.dt, fma_rn(p.Du, su, ru), luc);
-            out.v[e] = fma_rn(p.dt, fma_rn(p.Dv, sv, rv), lvc);
-            if (own) {
-                rg[0] = fma_rn(uc, fma_rn(T(-4), luc, su), rg[0]);     // u Lap(lu)
-                rg[1] = fma_rn(vc, fma_rn(T(-4), lvc, sv), rg[1]);     // v Lap(lv)
-                if (RX == RX_FHN) {
-                    rg[2] = add_rn(rg[2], lvc);                        // lv        (x -eps)
-                    rg[3] = fma_rn(lvc, vc, rg[3]);                    // lv v      (x eps)
-                    rg[4] = fma_rn(lvc, fma_rn(p.mb, vc, uc), rg[4]);  // lv (u - b v)
-                    rg[5] = fma_rn(luc, uc, rg[5]);                    // lu u
-                }
-            }
+            reverse_cell<T, RX>(B.u[e], B.v[e], nu[e], nv[e], flip ? stu[V - 1 - e] : stu[e],
+                                flip ? stv[V - 1 - e] : stv[e], p, own, rg, out.u[e], out.v[e]);
         }
     }
     __device__ __forceinline__ void finish(int q, const Slice<T> &out) {

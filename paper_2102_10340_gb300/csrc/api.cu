@@ -320,7 +320,7 @@ static bool ensure_graph(rdcnn_t *h, int variant, int k, void *su, void *sv) {
 // Most steps of one resident launch: 1 .. 7 ms.
 constexpr int64_t kResidentSteps = 8192;
 
-int run_core(rdcnn_t *h, int64_t T, int variant, int k, int64_t every, MarkFn mark, void *ctx) {
+int run_core(rdcnn_t *h, int64_t T, int variant, int k, int64_t every, MarkFn mark, void *ctx, DestFn dest) {
     if (!h) return set_error(RDCNN_EINVAL, "handle is NULL");
     if (!h->bound) return set_error(RDCNN_ESTATE, "handle is not bound");
     if (T < 0) return set_error(RDCNN_EINVAL, "T must be >= 0");
@@ -384,13 +384,28 @@ int run_core(rdcnn_t *h, int64_t T, int variant, int k, int64_t every, MarkFn ma
         int kk = (int)(left < k ? left : k);
         const int64_t done = T - left;
         if (every > 0) kk = (int)std::min<int64_t>(kk, every - done % every);
-        const cudaError_t e = launch_one(h, variant, kk, cu, cv, nu, nv, h->stream);
+        const bool marks = every > 0 && (done + kk) % every == 0;
+        void *du = nullptr, *dv = nullptr;
+        const bool straight = marks && dest && dest(ctx, done + kk, &du, &dv);
+        const cudaError_t e = launch_one(h, variant, kk, cu, cv, straight ? du : nu, straight ? dv : nv, h->stream);
         if (e != cudaSuccess) return cuda_error(e, "step kernel launch");
-        const void *tu = cu, *tv = cv;
-        cu = nu; cv = nv;
-        nu = const_cast<void *>(tu); nv = const_cast<void *>(tv);
+        if (straight) {
+            // both pairs are free now: the last launch but for marks ends in (u, v)
+            cu = du; cv = dv;
+            nu = su; nv = sv;
+            if (((left - kk + k - 1) / k) % 2 == 1) { nu = h->u; nv = h->v; }
+        } else {
+            const void *tu = cu, *tv = cv;
+            cu = nu; cv = nv;
+            if (tu == h->u || tu == su) {
+                nu = const_cast<void *>(tu); nv = const_cast<void *>(tv);
+            } else {  // tu was a mark's destination
+                nu = cu == h->u ? su : h->u;
+                nv = cu == h->u ? sv : h->v;
+            }
+        }
         left -= kk;
-        if (every > 0 && (T - left) % every == 0 && mark) {
+        if (marks && !straight && mark) {
             const int rc = mark(ctx, T - left, cu, cv);
             if (rc < 0) return rc;
         }

@@ -116,10 +116,15 @@ int handle_view(const rdcnn_t *h, int64_t *nn, int64_t *nm, rdcnn_params *p, int
 // multiple of `every`), with the planes that hold the state at that step.
 typedef int (*MarkFn)(void *ctx, int64_t t, const void *cu, const void *cv);
 
+// Planes of the caller's that shall hold the state at step t (a multiple of
+// `every`): the launch that completes step t then writes them itself, the next
+// one reads them, and mark is not called for t.  False: none for this t.
+typedef bool (*DestFn)(void *ctx, int64_t t, void **du, void **dv);
+
 // Advance the bound state of h by T steps (the body of rdcnn_run).  With
 // every > 0 no launch crosses a multiple of `every`, and mark(ctx, t, ...)
 // runs after each such step t.  Result in h->u, h->v.
-int run_core(rdcnn_t *h, int64_t T, int variant, int k, int64_t every, MarkFn mark, void *ctx);
+int run_core(rdcnn_t *h, int64_t T, int variant, int k, int64_t every, MarkFn mark, void *ctx, DestFn dest = nullptr);
 
 // Kernel launchers.  All return the launch status (cudaGetLastError()).
 // u/v are read, un/vn written; the two pairs must not overlap.  reaction is

@@ -342,7 +342,7 @@ int run_core(rdcnn_t *h, int64_t T, int variant, int k, int64_t every, MarkFn ma
     // ignores it.
     if (autov && variant == RDCNN_VARIANT_GENERIC && h->dtype == RDCNN_F32) {
         variant = kVariantRagged;
-        k = (k_arg >= 1 && k_arg <= max_k(h->dtype)) ? k_arg : h->tune_k ? h->tune_k : default_k(h->dtype, h->nn, h->nm);
+        k = (k_arg >= 1 && k_arg <= max_k(h->dtype)) ? k_arg : h->tune_k ? h->tune_k : default_k_ragged(h->nn, h->nm);
     }
     const void *cu = h->u, *cv = h->v;
     void *nu = su, *nv = sv;
@@ -365,6 +365,8 @@ int run_core(rdcnn_t *h, int64_t T, int variant, int k, int64_t every, MarkFn ma
         }
         if (left == 0) return RDCNN_OK;
     }
+    // FP32 bits do not depend on the depth of a launch: without one asked for, it is free
+    const bool own_depth = autov && k_arg == 0 && h->tune_k == 0 && h->dtype == RDCNN_F32;
     // launch-bound runs: replay whole groups of full-depth launches as a graph
     const int64_t full = left / k;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -384,6 +386,14 @@ int run_core(rdcnn_t *h, int64_t T, int variant, int k, int64_t every, MarkFn ma
         int kk = (int)(left < k ? left : k);
         const int64_t done = T - left;
         if (every > 0) kk = (int)std::min<int64_t>(kk, every - done % every);
+        if (own_depth) {
+            // the launches up to the end or the next mark, of even depth rather than
+            // full ones and a rest; up to the end, as many as end in (u, v)
+            const int64_t stretch = every > 0 ? std::min<int64_t>(left, every - done % every) : left;
+            int64_t n = (stretch + k - 1) / k;
+            if (every == 0 && (n % 2 == 0) != (cu == h->u) && n < stretch) ++n;
+            kk = (int)((stretch + n - 1) / n);
+        }
         const bool marks = every > 0 && (done + kk) % every == 0;
         void *du = nullptr, *dv = nullptr;
         const bool straight = marks && dest && dest(ctx, done + kk, &du, &dv);

@@ -206,8 +206,76 @@ cudaError_t step1_t(int reaction, int boundary, const void *u, const void *v, vo
 
 }  // namespace
 
-// Rows per warp strip when the caller gives none.  Small grids use short
-// strips (few warps exist at all); large grids pick, among a few lengths,
+// Launch shape of the FP32 temporal pipeline, rows per warp and depth, from a
+// model of a launch: a warp's strip of R rows is R beats and a fill of f k more,
+// and a beat takes a + b k us with one warp on each of an SM's four schedulers,
+// a2 + b2 k with two (which is what the registers of k = 8 allow); more warps
+// run in waves of that.  So only a few strip lengths can be best for a depth:
+// those with which the warps just fill one warp per scheduler, two, or w waves.
+// Fitted (us) to a sweep of k = 3 .. 8 and 25 strip lengths at 18 shapes from
+// 300^2 to 4096^2, FitzHugh-Nagumo on the torus and under zero flux, CeNN under
+// zero flux: the shape it picks is within 1.1 % of the best one measured (7 % at
+// most), the size classes before it (k = 4, 6, 8; 4 or 16 rows below 2^22 cells)
+// were 17 % off on average and up to 68 %.  us a step, before / now: 384^2
+// 1.18 / 0.95, 768^2 1.51 / 1.30, 1536^2 3.47 / 2.45, 3072^2 8.03 / 6.33, 4096 x
+// 1024 4.56 / 3.62, 1024^2 and 4096^2 unchanged.  Ragged rows cost more per beat
+// (single elements are copied), so their depths begin at 5: 14 shapes, 3.2 % off
+// the best on average (13 % at most), before 22 %.
+namespace {
+
+struct BeatModel {
+    double launch, a, b, f, a2, b2, f2;
+    int k0, k1;  // depths AUTO chooses among
+};
+constexpr BeatModel kBeats = {1.680, 0.0764, 0.0394, 2.690, 0.0692, 0.0548, 1.823, 4, 8};
+constexpr BeatModel kRaggedBeats = {1.692, 0.2179, 0.0290, 3.830, 0.1335, 0.0829, 1.714, 5, 8};
+
+// us of a launch of depth K with `warps` strips of `rows` rows.
+double launch_us(const BeatModel &m, int K, int64_t warps, int64_t rows, int64_t slots) {
+    if (warps <= slots / 2) return m.launch + (m.a + m.b * K) * ((double)rows + m.f * K);
+    return m.launch + (double)((warps + slots - 1) / slots) * (m.a2 + m.b2 * K) * ((double)rows + m.f2 * K);
+}
+
+// Best rows for depth K; *us: what a launch then takes.
+int model_rows(const BeatModel &m, int K, int64_t nn, int64_t nm, double *us) {
+    const int H = (K + 3) / 4;
+    const int64_t bands = (nm + (32 - 2 * H) * 4 - 1) / ((32 - 2 * H) * 4);
+    const int64_t slots = (int64_t)sm_count() * 8;
+    int best = 1;
+    *us = 1e300;
+    for (int w = 0; w <= 8; ++w) {  // w = 0: one warp per scheduler
+        const int64_t strips = std::min<int64_t>((w ? w * slots : slots / 2) / bands, (nn + 1) / 2);
+        if (strips < 1) continue;
+        const int64_t rows = (nn + strips - 1) / strips;
+        const double t = launch_us(m, K, bands * ((nn + rows - 1) / rows), rows, slots);
+        if (t < *us) { *us = t; best = (int)rows; }
+    }
+    if (*us > 1e299) best = 256;  // more bands than the waves looked at hold
+    return best;
+}
+
+int model_depth(const BeatModel &m, int64_t nn, int64_t nm) {
+    int best = m.k1;
+    double least = 1e300;
+    for (int K = m.k0; K <= m.k1; ++K) {
+        double us;
+        (void)model_rows(m, K, nn, nm, &us);
+        if (us / K < least) { least = us / K; best = K; }
+    }
+    return best;
+}
+
+}  // namespace
+
+double temporal_us(int K, int64_t warps, int64_t rows) { return launch_us(kBeats, K, warps, rows, (int64_t)sm_count() * 8); }
+
+int auto_rows_f32(bool ragged, int K, int64_t nn, int64_t nm) {
+    double us;
+    return model_rows(ragged ? kRaggedBeats : kBeats, K, nn, nm, &us);
+}
+
+// Rows per warp strip when the caller gives none (FP64 and 16-bit planes, 8
+// values per lane, warp pairs).  Small grids use short strips (few warps exist at all); large grids pick, among a few lengths,
 // the one that minimises waves x (rows + 2K) -- the work of the slowest SM
 // when every resident warp slot is busy -- so a launch does not spill a
 // nearly empty second wave (e.g. 4096^2, K=8: 128 rows = 1184 warps, one
@@ -382,19 +450,20 @@ int plan_rows(int dtype, int reaction, int boundary, int variant, int k, int64_t
     return out;
 }
 
-// Temporal depth by grid size, from a launch-shape sweep on GB300 (FP32,
-// square grids): 128^2-256^2 k=4, 512^2 k=6, 1024^2 k=4, >= 2048^2 k=8.
-// Small grids are latency/launch bound, where fewer, shallower stages in
-// more warps win; large grids are FP32-pipe bound, where depth amortises
-// the halo.  FP64: 2, see auto_single_step.
+// Temporal depth when the caller gives none.  FP32: the model above.  FP64: 2,
+// see auto_single_step.  16-bit planes round once per launch, so the depth is
+// part of their result: by size class, k = 4 below 2^17 cells, 6 below 2^19, 4
+// below 2^21, 8 above.
 int default_k(int dtype, int64_t nn, int64_t nm) {
     const int64_t cells = nn * nm;
     if (dtype == RDCNN_F64) return 2;
+    if (dtype == RDCNN_F32) return model_depth(kBeats, nn, nm);
     if (cells >= (int64_t(1) << 21)) return 8;
     if (cells >= (int64_t(1) << 19)) return 4;
     if (cells >= (int64_t(1) << 17)) return 6;
     return 4;
 }
+int default_k_ragged(int64_t nn, int64_t nm) { return model_depth(kRaggedBeats, nn, nm); }
 
 // FP64 runs at 1/64 of the FP32 rate, so the FP64 pipe bounds every grid that
 // fills the GPU, and a halo cell costs as much as an owned one: the single

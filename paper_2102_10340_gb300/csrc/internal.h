@@ -177,6 +177,10 @@ int plan_rows(int dtype, int reaction, int boundary, int variant, int k, int64_t
 // Rows per warp strip of a temporal launch (wave-quantisation model).
 int auto_rows_temporal(int K, int64_t nn, int64_t nm, int bands, int blocks_per_sm,
                        int warps_per_block);
+// The same for FP32 planes with 4 values per lane (launch model in forward.cu).
+int auto_rows_f32(bool ragged, int K, int64_t nn, int64_t nm);
+// us of an FP32 temporal launch of depth K with that many strips of that many rows.
+double temporal_us(int K, int64_t warps, int64_t rows);
 // u = v = ka * x; x may alias u.
 cudaError_t launch_init(int dtype, const void *x, void *u, void *v, double ka, int64_t n,
                         cudaStream_t s);
@@ -185,6 +189,7 @@ cudaError_t launch_init(int dtype, const void *x, void *u, void *v, double ka, i
 // itself when given rows <= 0.
 int default_rows_step1(int dtype, int64_t nn, int64_t nm);
 int default_k(int dtype, int64_t nn, int64_t nm);
+int default_k_ragged(int64_t nn, int64_t nm);
 // Whether AUTO takes the single-step kernel rather than a temporal depth.
 bool auto_single_step(int dtype);
 

@@ -33,6 +33,7 @@ constexpr int temporal_bands(int64_t nm) {
 template <typename T, int K>
 int temporal_rows(int reaction, int boundary, int64_t nn, int64_t nm, int rows) {
     if (rows > 0) return rows;
+    if constexpr (std::is_same<T, float>::value || IsRagged<T>::value) return auto_rows_f32(IsRagged<T>::value, K, nn, nm);
     int r = 0;
     with_model(reaction, boundary, [&](auto rx, auto bc) {
         r = auto_rows_temporal(K, nn, nm, temporal_bands<T, K>(nm),

@@ -1,0 +1,77 @@
+"""Launch shapes and stretches that AUTO chooses: runs end in (u, v) whatever the number of launches,
+device snapshots written by the steps themselves, statistics with and without whole vectors, and FP32
+batches of mixed sizes, each against the plain path."""
+import numpy as np
+import pytest
+import torch
+
+import rdcnn_inputs as inp
+from _util import gpu_run
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("shape", [(2, 260), (45, 300), (301, 299), (700, 264), (1030, 520)])
+@pytest.mark.parametrize("boundary", ["periodic", "zeroflux"])
+def test_any_number_of_steps(rd, shape, boundary):
+    x, y = inp.uniform_field(71, *shape), 0.7 * inp.uniform_field(72, *shape)
+    for T in (1, 2, 3, 5, 8, 9, 17, 41):
+        a, b = (gpu_run(rd, x, y, inp.default_params(), T, torch.float32, v, boundary=boundary) for v in ("auto", "generic"))
+        assert (a[0] == b[0]).all() and (a[1] == b[1]).all(), T
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64, torch.bfloat16])
+@pytest.mark.parametrize("shape", [(96, 300), (64, 64), (37, 261)])
+@pytest.mark.parametrize("T,every", [(20, 20), (23, 7), (12, 1), (5, 9), (30, 4)])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_device_snapshots(rd, dtype, shape, T, every, offset):
+    """Against copies of the state taken between runs of `every` steps (16-bit: the same launches).
+    offset: the arrays one element off an aligned address."""
+    n = T // every + 1
+    g = rd.Grid(*shape, inp.default_params(), dtype=dtype)
+    x = torch.from_numpy(inp.uniform_field(73, *shape)).to(dtype).cuda()
+    g.init(x)
+    cells = n * shape[0] * shape[1]
+    base = [torch.full((cells + 2,), 7.0, dtype=dtype, device="cuda") for _ in range(2)]
+    us, vs = (t[offset:offset + cells].view(n, *shape) for t in base)
+    g.run_snapshots(T, every, out="device", buffers=(us, vs))
+    h = rd.Grid(*shape, inp.default_params(), dtype=dtype)
+    h.init(x)
+    for s in range(n):
+        assert torch.equal(us[s], h.u) and torch.equal(vs[s], h.v), s
+        h.run(every if s + 1 < n else T % every)
+    assert torch.equal(g.u, h.u) and torch.equal(g.v, h.v)
+    assert all(float(t[-1]) == 7.0 and (offset == 0 or float(t[0]) == 7.0) for t in base)
+
+
+@pytest.mark.parametrize("shape", [(1, 4), (9, 124), (16, 128), (1000, 132), (5, 131), (70, 516)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64, torch.float16])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_statistics_with_and_without_vectors(rd, shape, dtype, offset):
+    """FP32 sums of up to 16 values a lane and 8 lanes' tree: 1e-5 relative, FP64 1e-12."""
+    cells = shape[0] * shape[1]
+    base = [torch.zeros(cells + 1, dtype=dtype, device="cuda") for _ in range(2)]
+    u, v = (t[offset:offset + cells].view(shape) for t in base)
+    u.copy_(torch.from_numpy(inp.uniform_field(74, *shape)))
+    v.copy_(torch.from_numpy(inp.uniform_field(75, *shape)))
+    got = rd.rdcnn.grid_summary(u, v, 0.8).numpy() if hasattr(rd, "rdcnn") else rd.grid_summary(u, v, 0.8).numpy()
+    a, b = u.double().cpu().numpy(), v.double().cpu().numpy()
+    grad = np.abs(np.roll(a, -1, 0) - a) + np.abs(np.roll(a, -1, 1) - a)
+    want = [a.mean(), a.var(), a.min(), a.max(), b.mean(), b.var(), grad.mean(), (grad > 0.8).mean()]
+    tol = 1e-12 if dtype == torch.float64 else 1e-5
+    np.testing.assert_allclose(got[:7], want[:7], rtol=tol, atol=tol)
+    assert abs(got[7] - want[7]) <= 2.0 / cells  # a gradient within rounding of the threshold
+
+
+@pytest.mark.parametrize("sides", [(32,), (32, 300), (128, 256, 512), (64, 1024, 96)])
+@pytest.mark.parametrize("T", [1, 3, 16, 29])
+def test_batches_of_mixed_sizes(rd, sides, T):
+    specs = [{"nn": s, "nm": s + 4 * i, "params": inp.default_params(Du=0.03 * (i + 1))} for i, s in enumerate(sides * 2)]
+    b = rd.Batch(specs, dtype=torch.float32)
+    xs = [torch.from_numpy(inp.uniform_field(76 + i, s["nn"], s["nm"])).float().cuda() for i, s in enumerate(specs)]
+    for i, x in enumerate(xs):
+        b.set_state(i, x, -x)
+    b.run(T)
+    for i, (s, x) in enumerate(zip(specs, xs)):
+        ref = gpu_run(rd, x.double().cpu().numpy(), -x.double().cpu().numpy(), s["params"], T, torch.float32, "generic")
+        assert all((t.cpu().numpy() == r).all() for t, r in zip(b.state(i), ref)), i

@@ -254,6 +254,13 @@ typedef struct rdcnn_instance {
     void *su, *sv;
 } rdcnn_instance;
 
+/* Copy a state (planes u0, v0 of `bytes` each, which may be the same) into an
+ * instance's planes u, v, all device memory, asynchronously on `stream`: one
+ * kernel where the planes are 16-byte aligned, whole multiples of 16 bytes and
+ * disjoint, otherwise u first, then v.  Errors: RDCNN_EINVAL (NULL),
+ * RDCNN_ECUDA. */
+int rdcnn_copy_state(void *u, void *v, const void *u0, const void *v0, size_t bytes, void *stream);
+
 /* Bytes of device workspace rdcnn_batch_run needs for its work table. */
 int rdcnn_batch_workspace_bytes(const rdcnn_instance *inst, int n, int dtype,
                                 const rdcnn_tune *tune, size_t *bytes);

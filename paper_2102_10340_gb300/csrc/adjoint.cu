@@ -392,8 +392,7 @@ int reverse_sweep(rdcnn_t *h, int64_t nn, int64_t nm, const rdcnn_params &p, int
     if (single) partial = (double *)(ws + L.seg_off);
     const size_t partial_bytes = single ? one.bytes : (size_t)sh.nwarps * 6 * sizeof(double);
 
-    cudaError_t e = cudaMemcpyAsync(lam_u[0], dLdu_T, bytes, cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(lam_v[0], dLdv_T, bytes, cudaMemcpyDeviceToDevice, s);
+    cudaError_t e = copy_planes(lam_u[0], lam_v[0], dLdu_T, dLdv_T, bytes, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(partial, 0, partial_bytes, s);
     if (e != cudaSuccess) return cuda_error(e, "adjoint setup copies");
     if (overlap) {  // the rebuilds read the checkpoints
@@ -469,8 +468,7 @@ int reverse_sweep(rdcnn_t *h, int64_t nn, int64_t nm, const rdcnn_params &p, int
     count_launches(1);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_error(e, "gradient reduction");
-    e = cudaMemcpyAsync(dLdu0, lam_u[cur], bytes, cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(dLdv0, lam_v[cur], bytes, cudaMemcpyDeviceToDevice, s);
+    e = copy_planes(dLdu0, dLdv0, lam_u[cur], lam_v[cur], bytes, s);
     double hg[6];
     if (e == cudaSuccess) e = cudaMemcpyAsync(hg, gout, sizeof(hg), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -491,8 +489,7 @@ int adjoint_t(rdcnn_t *h, int64_t nn, int64_t nm, const rdcnn_params &p, int dty
               const void *dLdv_T, const AdjLayout &L, char *ws, void *dLdu0, void *dLdv0, double grad[6]) {
     const size_t bytes = (size_t)nn * nm * sizeof(T);
     char *ck = ws + L.ck_off;
-    cudaError_t e = cudaMemcpyAsync(ck, u0, bytes, cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(ck + L.plane, v0, bytes, cudaMemcpyDeviceToDevice, s);
+    cudaError_t e = copy_planes(ck, ck + L.plane, u0, v0, bytes, s);
     if (e != cudaSuccess) return cuda_error(e, "adjoint setup copies");
     // a co-state plane pair serves as the sweep's scratch until the reverse sweep starts
     char *lam = ws + L.lam_off;
@@ -583,8 +580,7 @@ int rdcnn_run_record(rdcnn_t *h, int64_t T, int64_t n_checkpoints, void *tape, s
     if (tape_bytes < L.tape) return set_error(RDCNN_ESPACE, "tape has %zu bytes, need %zu", tape_bytes, L.tape);
     const size_t bytes = (size_t)nn * nm * elem_size(dtype);
     char *ck = (char *)tape;
-    cudaError_t e = cudaMemcpyAsync(ck, h->u, bytes, cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(ck + L.plane, h->v, bytes, cudaMemcpyDeviceToDevice, s);
+    cudaError_t e = copy_planes(ck, ck + L.plane, h->u, h->v, bytes, s);
     if (e != cudaSuccess) return cuda_error(e, "tape slot 0");
     if (T == 0) return RDCNN_OK;
     // scratch: the bound ping-pong planes (second one at the rounded stride)

@@ -172,10 +172,14 @@ int rdcnn_set_state(rdcnn_t *h, const void *u0, const void *v0, int on_device) {
     if (!h->bound) return set_error(RDCNN_ESTATE, "handle is not bound");
     if (!u0 || !v0) return set_error(RDCNN_EINVAL, "state pointer is NULL");
     const size_t bytes = (size_t)h->nn * h->nm * elem_size(h->dtype);
-    const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    cudaError_t e = cudaMemcpyAsync(h->u, u0, bytes, kind, h->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h->v, v0, bytes, kind, h->stream);
-    if (e == cudaSuccess && !on_device) e = cudaStreamSynchronize(h->stream);
+    cudaError_t e;
+    if (on_device) {
+        e = copy_planes(h->u, h->v, u0, v0, bytes, h->stream);
+    } else {
+        e = cudaMemcpyAsync(h->u, u0, bytes, cudaMemcpyHostToDevice, h->stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(h->v, v0, bytes, cudaMemcpyHostToDevice, h->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    }
     if (e != cudaSuccess) return cuda_error(e, "set_state copy");
     return RDCNN_OK;
 }
@@ -421,8 +425,7 @@ int run_core(rdcnn_t *h, int64_t T, int variant, int k, int64_t every, MarkFn ma
         }
     }
     if (cu != h->u) {
-        cudaError_t e = cudaMemcpyAsync(h->u, cu, plane, cudaMemcpyDeviceToDevice, h->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(h->v, cv, plane, cudaMemcpyDeviceToDevice, h->stream);
+        const cudaError_t e = copy_planes(h->u, h->v, cu, cv, plane, h->stream);
         if (e != cudaSuccess) return cuda_error(e, "copy back to state");
     }
     return RDCNN_OK;

@@ -182,6 +182,12 @@ using namespace rdk;
 
 extern "C" {
 
+int rdcnn_copy_state(void *u, void *v, const void *u0, const void *v0, size_t bytes, void *stream) {
+    if (!u || !v || !u0 || !v0) return set_error(RDCNN_EINVAL, "NULL plane");
+    const cudaError_t e = copy_planes(u, v, u0, v0, bytes, (cudaStream_t)stream);
+    return e == cudaSuccess ? RDCNN_OK : cuda_error(e, "copy state");
+}
+
 int rdcnn_batch_workspace_bytes(const rdcnn_instance *inst, int n, int dtype,
                                 const rdcnn_tune *tune, size_t *bytes) {
     (void)inst; (void)dtype; (void)tune;

@@ -185,6 +185,11 @@ double temporal_us(int K, int64_t warps, int64_t rows);
 cudaError_t launch_init(int dtype, const void *x, void *u, void *v, double ka, int64_t n,
                         cudaStream_t s);
 
+// Whether kernels of the current device may use p: its own or managed memory.
+bool on_this_device(const void *p);
+// du = su and dv = sv, `bytes` each, device memory.
+cudaError_t copy_planes(void *du, void *dv, const void *su, const void *sv, size_t bytes, cudaStream_t s);
+
 // Default launch shapes.  launch_temporal picks its rows per warp strip
 // itself when given rows <= 0.
 int default_rows_step1(int dtype, int64_t nn, int64_t nm);

@@ -27,6 +27,7 @@ struct SnapCtx {
     size_t plane = 0;
     char *u_snap = nullptr, *v_snap = nullptr;
     bool on_device = false;
+    bool direct = false;  // the kernels can write the arrays
     char *staging = nullptr;
     int n_stage = 0;
     std::vector<cudaEvent_t> ready, freed;
@@ -36,9 +37,7 @@ int take_snapshot(SnapCtx &c, int64_t s, const void *cu, const void *cv) {
     rdcnn_t *h = c.h;
     cudaError_t e;
     if (c.on_device) {
-        e = cudaMemcpyAsync(c.u_snap + s * c.plane, cu, c.plane, cudaMemcpyDeviceToDevice, h->stream);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(c.v_snap + s * c.plane, cv, c.plane, cudaMemcpyDeviceToDevice, h->stream);
+        e = copy_planes(c.u_snap + s * c.plane, c.v_snap + s * c.plane, cu, cv, c.plane, h->stream);
         return e == cudaSuccess ? RDCNN_OK : cuda_error(e, "snapshot copy");
     }
     const int slot = (int)(s % c.n_stage);
@@ -46,8 +45,7 @@ int take_snapshot(SnapCtx &c, int64_t s, const void *cu, const void *cv) {
     char *sv = su + c.plane;
     e = cudaSuccess;
     if (s >= c.n_stage) e = cudaStreamWaitEvent(h->stream, c.freed[slot], 0);  // slot's last host copy done
-    if (e == cudaSuccess) e = cudaMemcpyAsync(su, cu, c.plane, cudaMemcpyDeviceToDevice, h->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(sv, cv, c.plane, cudaMemcpyDeviceToDevice, h->stream);
+    if (e == cudaSuccess) e = copy_planes(su, sv, cu, cv, c.plane, h->stream);
     if (e == cudaSuccess) e = cudaEventRecord(c.ready[slot], h->stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(h->copy_stream, c.ready[slot], 0);
     if (e == cudaSuccess)
@@ -65,10 +63,10 @@ int on_mark(void *ctx, int64_t t, const void *cu, const void *cv) {
 
 // Device snapshots: the launch that completes the step writes the slot (768 x
 // 1024, every 20 of 200 steps: 493 -> 420 us against a pair of copies per slot).  Slots
-// off the vectorised kernels' alignment are copied to.
+// off the vectorised kernels' alignment, and arrays on another device, are copied to.
 bool snapshot_planes(void *ctx, int64_t t, void **du, void **dv) {
     SnapCtx &c = *static_cast<SnapCtx *>(ctx);
-    if (!c.on_device) return false;
+    if (!c.direct) return false;
     *du = c.u_snap + t / c.every * c.plane;
     *dv = c.v_snap + t / c.every * c.plane;
     return aligned16(*du) && aligned16(*dv);
@@ -95,6 +93,7 @@ int rdcnn_run_snapshots(rdcnn_t *h, int64_t T, int64_t every, void *u_snap, void
     c.u_snap = (char *)u_snap;
     c.v_snap = (char *)v_snap;
     c.on_device = snap_on_device != 0;
+    c.direct = c.on_device && on_this_device(u_snap) && on_this_device(v_snap);
     if (!c.on_device) {
         c.staging = (char *)staging;
         c.n_stage = staging ? (int)std::min<size_t>(staging_bytes / (2 * c.plane), 1 << 16) : 0;

@@ -82,6 +82,10 @@ class Grid:
 
     def __init__(self, nn: int, nm: int, params: dict | None = None, dtype=torch.float32,
                  reaction: str = "fhn", device="cuda", boundary: str = "periodic"):
+        self._open(nn, nm, params, dtype, reaction, device, boundary, torch.zeros)
+
+    def _open(self, nn, nm, params, dtype, reaction, device, boundary, planes):
+        """planes: torch.zeros, or torch.empty where the state is set before anything reads it."""
         self.lib = L.load()
         self.nn, self.nm = int(nn), int(nm)
         self.dtype = dtype
@@ -98,8 +102,8 @@ class Grid:
         self.h = h
         nbytes = ctypes.c_size_t()
         L.check(self.lib.rdcnn_workspace_bytes(self.h, ctypes.byref(nbytes)))
-        self.u = torch.zeros((self.nn, self.nm), dtype=dtype, device=self.device)
-        self.v = torch.zeros((self.nn, self.nm), dtype=dtype, device=self.device)
+        self.u = planes((self.nn, self.nm), dtype=dtype, device=self.device)
+        self.v = planes((self.nn, self.nm), dtype=dtype, device=self.device)
         esz = torch.finfo(dtype).bits // 8
         self.workspace = torch.empty(nbytes.value // esz, dtype=dtype, device=self.device)
         self._bind()
@@ -385,8 +389,15 @@ class Batch:
         return sum(it["nn"] * it["nm"] for it in self.items)
 
     def set_state(self, i: int, u0, v0):
-        self.items[i]["u"].copy_(torch.as_tensor(u0, dtype=self.dtype))
-        self.items[i]["v"].copy_(torch.as_tensor(v0, dtype=self.dtype))
+        it = self.items[i]
+        u, v = it["u"], it["v"]
+        if all(type(t) is torch.Tensor and t.dtype == self.dtype and t.device == u.device and t.shape == u.shape
+               and t.is_contiguous() and not t.requires_grad for t in (u0, v0)):
+            L.check(self.lib.rdcnn_copy_state(u.data_ptr(), v.data_ptr(), u0.data_ptr(), v0.data_ptr(),
+                                              u.numel() * u.element_size(), _stream_ptr(u.device)))
+            return
+        u.copy_(torch.as_tensor(u0, dtype=self.dtype))
+        v.copy_(torch.as_tensor(v0, dtype=self.dtype))
 
     def set_tune(self, k: int = 0, rows: int = 0):
         self.tune = L.Tune(int(k), int(rows))
@@ -454,11 +465,13 @@ class RDCNNFunction(torch.autograd.Function):
         th = [float(x) for x in theta.detach().cpu().tolist()]
         params = dict(zip(GRAD_NAMES, th))
         params["dt"] = float(dt)
-        g = Grid(u0.shape[0], u0.shape[1], params, dtype=u0.dtype, device=u0.device, boundary=boundary,
-                 reaction=reaction)
+        g = Grid.__new__(Grid)
+        g._open(u0.shape[0], u0.shape[1], params, u0.dtype, reaction, u0.device, boundary, torch.empty)
         g.set_state(u0.detach(), v0.detach())
         ctx.tape = g.run_record(int(T), int(n_checkpoints))
-        uT, vT = g.state()
+        # the grid is this call's own: its planes are the results, and backward reads only the tape
+        uT, vT = g.u, g.v
+        g.u, g.v = uT.detach(), vT.detach()
         ctx.save_for_backward(u0.detach(), v0.detach())
         ctx.grid = g
         ctx.T = int(T)

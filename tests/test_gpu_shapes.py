@@ -75,3 +75,42 @@ def test_batches_of_mixed_sizes(rd, sides, T):
     for i, (s, x) in enumerate(zip(specs, xs)):
         ref = gpu_run(rd, x.double().cpu().numpy(), -x.double().cpu().numpy(), s["params"], T, torch.float32, "generic")
         assert all((t.cpu().numpy() == r).all() for t, r in zip(b.state(i), ref)), i
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64, torch.bfloat16])
+def test_batch_state_copies(rd, dtype):
+    """States from tensors of every kind a caller may hold: the same plane twice, whole and offset
+    views, another type, transposed, on the host, and the instance's own planes (u is set first)."""
+    nn, nm = 33, 52
+    specs = [{"nn": nn, "nm": nm, "params": inp.default_params()}]
+    x, y = (torch.from_numpy(inp.uniform_field(s, nn, nm)).to(dtype).cuda() for s in (81, 82))
+    off = torch.zeros(nn * nm + 1, dtype=dtype, device="cuda")[1:].view(nn, nm)
+    off.copy_(y)
+    for a, b in ((x, x), (x, y), (x, off), (off, x), (x.double(), y.float()), (x, y.t().contiguous().t()), (x.cpu(), y.cpu())):
+        t = rd.Batch(specs, dtype=dtype)
+        t.set_state(0, a, b)
+        assert torch.equal(t.state(0)[0], a.to("cuda", dtype)) and torch.equal(t.state(0)[1], b.to("cuda", dtype))
+    t.set_state(0, x, y)
+    t.set_state(0, t.state(0)[1], t.state(0)[0])
+    assert torch.equal(t.state(0)[0], y) and torch.equal(t.state(0)[1], y)
+    with pytest.raises(RuntimeError):
+        t.set_state(0, x[:, :-4].contiguous(), y[:, :-4].contiguous())
+
+
+def test_training_results_outlive_later_calls(rd):
+    """The final state returned by RDCNNFunction keeps its values, and the graph its gradients, when
+    the outputs are written over and other calls run in between."""
+    f = lambda seed: torch.from_numpy(inp.uniform_field(seed, 40, 64)).float().cuda()  # noqa: E731
+    th = torch.tensor([inp.default_params()[k] for k in rd.GRAD_NAMES], dtype=torch.float64)
+    out = []
+    for disturb in (False, True):
+        u0, v0, t = f(91).requires_grad_(True), f(92).requires_grad_(True), th.clone().requires_grad_(True)
+        u, v = rd.RDCNNFunction.apply(u0, v0, t, 30)
+        loss = (u * f(93)).sum() + (v * f(94)).sum()
+        kept = u.detach().clone()
+        if disturb:
+            with torch.no_grad():
+                rd.RDCNNFunction.apply(f(95), f(96), th, 7)
+                u.detach().zero_()
+        out.append((kept, *torch.autograd.grad(loss, (u0, v0, t))))
+    assert all(torch.equal(a, b) for a, b in zip(*out))

@@ -273,8 +273,10 @@ int rdcnn_batch_workspace_bytes(const rdcnn_instance *inst, int n, int dtype,
  * layout rules as for rdcnn_run apply to every instance (NM a multiple of 4,
  * or 2 for F64; 16-byte aligned pointers, 8-byte for BF16 / F16), else
  * RDCNN_EINVAL.  tune may be NULL.
- * Asynchronous on `stream`, except that the work table is copied to the
- * device first (host-synchronous copy into `workspace`). */
+ * Asynchronous on `stream`, except that the work table of more than 64
+ * instances, or of planes other than F32, is copied to the device first
+ * (host-synchronous copy into `workspace`).  Not while `stream` is being
+ * captured (RDCNN_ECUDA). */
 int rdcnn_batch_run(const rdcnn_instance *inst, int n, int64_t T, int dtype, int reaction,
                     const rdcnn_tune *tune, void *workspace, size_t workspace_bytes,
                     void *stream);

@@ -5,7 +5,8 @@
 // The host lays the instances out as a table of descriptors in device memory
 // with a running warp offset: instance i owns warps
 // [warp_begin_i, warp_begin_i + bands_i * strips_i).  A warp finds its instance
-// by binary search over warp_begin, then runs the same K-stage register
+// by binary search over warp_begin (FP32 batches of up to 64 instances: in a
+// table among the launch's parameters), then runs the same K-stage register
 // pipeline as the single-grid temporal kernel (temporal.cuh) with that
 // instance's gene.  All launches of one call use the same halo width H (the
 // one the deepest launch needs), so one table serves launches of any depth.
@@ -32,6 +33,9 @@
 RDK_EXTERN_BATCH_32(float)
 RDK_EXTERN_BATCH_32(__nv_bfloat16)
 RDK_EXTERN_BATCH_32(__half)
+RDK_EXTERN_BATCH_PARAM(1, 1) RDK_EXTERN_BATCH_PARAM(2, 1) RDK_EXTERN_BATCH_PARAM(3, 1) RDK_EXTERN_BATCH_PARAM(4, 1)
+RDK_EXTERN_BATCH_PARAM(1, 2) RDK_EXTERN_BATCH_PARAM(2, 2) RDK_EXTERN_BATCH_PARAM(3, 2) RDK_EXTERN_BATCH_PARAM(4, 2)
+RDK_EXTERN_BATCH_PARAM(5, 2) RDK_EXTERN_BATCH_PARAM(6, 2) RDK_EXTERN_BATCH_PARAM(7, 2) RDK_EXTERN_BATCH_PARAM(8, 2)
 RDK_EXTERN_BATCH(double, 1, 1) RDK_EXTERN_BATCH(double, 2, 1)
 RDK_EXTERN_BATCH(double, 1, 2) RDK_EXTERN_BATCH(double, 2, 2) RDK_EXTERN_BATCH(double, 3, 2)
 RDK_EXTERN_BATCH(double, 4, 2)
@@ -61,6 +65,17 @@ cudaError_t batch_launch(int dtype, int reaction, int boundary, int k, int H, co
         using T = decltype(tag);
         if (H == 1) return batch_launch_h<T, 1>(reaction, boundary, k, tab, n, nwarps, flip, s);
         return batch_launch_h<T, 2>(reaction, boundary, k, tab, n, nwarps, flip, s);
+    });
+}
+
+// k <= 4 H <= 8, as the caller has it.
+cudaError_t batch_param(int reaction, int boundary, int k, int H, const BatchParams &tab, unsigned nwarps, int flip,
+                        cudaStream_t s) {
+    return with_depth(k, [&](auto kk) -> cudaError_t {
+        constexpr int K = decltype(kk)::value;
+        if (H == 2) return batch_param_launch<K, 2>(reaction, boundary, tab, nwarps, flip, s);
+        if constexpr (K <= 4) return batch_param_launch<K, 1>(reaction, boundary, tab, nwarps, flip, s);
+        else return cudaErrorInvalidValue;
     });
 }
 
@@ -239,14 +254,30 @@ int rdcnn_batch_run_model(const rdcnn_instance *inst, int n, int64_t T, int dtyp
         d.dt = q.dt; d.Du = q.Du; d.Dv = q.Dv; d.cm4 = q.cm4;
         d.mthird = q.mthird; d.meps = q.meps; d.ebm4 = q.ebm4; d.mepsa = q.mepsa;
     }
-    cudaError_t e = cudaMemcpyAsync(workspace, tab.data(), n * sizeof(BatchDesc),
-                                    cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // host table goes out of scope
-    if (e != cudaSuccess) return cuda_error(e, "copy batch table");
+    // a few instances' table goes with each launch
+    const bool param = dtype == RDCNN_F32 && n <= kParamInstances && warps < (1ll << 31);
+    BatchParams ptab;
+    cudaError_t e = cudaSuccess;
+    if (param) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        e = cudaStreamIsCapturing(s, &cap);
+        if (e == cudaSuccess && cap != cudaStreamCaptureStatusNone) e = cudaErrorStreamCaptureUnsupported;  // as with the table's copy
+        if (e != cudaSuccess) return cuda_error(e, "batch run");
+        ptab.n = n;
+        for (int i = 0; i < n; ++i)
+            ptab.d[i] = BatchParam{(const float *)tab[i].u, (const float *)tab[i].v, (float *)tab[i].su, (float *)tab[i].sv,
+                                   tab[i].nn, tab[i].nm, tab[i].bands, tab[i].rows, (unsigned)tab[i].warp_begin,
+                                   make_coef<float>(inst[i].params, reaction)};
+    } else {
+        e = cudaMemcpyAsync(workspace, tab.data(), n * sizeof(BatchDesc), cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // host table goes out of scope
+        if (e != cudaSuccess) return cuda_error(e, "copy batch table");
+    }
     const std::vector<int> depths = dtype == RDCNN_F32 ? even_depths(T, k) : plan_depths(T, k);
     int flip = 0;
     for (int kk : depths) {
-        e = batch_launch(dtype, reaction, boundary, kk, H, (const BatchDesc *)workspace, n, warps, flip, s);
+        e = param ? batch_param(reaction, boundary, kk, H, ptab, (unsigned)warps, flip, s)
+                  : batch_launch(dtype, reaction, boundary, kk, H, (const BatchDesc *)workspace, n, warps, flip, s);
         if (e != cudaSuccess) return cuda_error(e, "batch kernel launch");
         flip ^= 1;
     }

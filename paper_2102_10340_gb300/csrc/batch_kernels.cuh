@@ -49,6 +49,55 @@ k_batch_temporal(const BatchDesc *__restrict__ tab, int n, long long nwarps, int
     pdl_trigger();
 }
 
+// FP32 batches of up to kParamInstances: the table travels with the launch, in
+// the constant bank.  The block's instance is found by a uniform search and its
+// gene stays in constant or uniform operands as in the single-grid kernel,
+// where the table in global memory puts it into eight registers of every
+// thread, whose bank conflicts and spills the pipeline pays for at every
+// instruction; nothing is copied to the device and waited for.  us a step, table
+// in memory / here: 24 instances of 128^2 .. 1024^2 7.71 / 7.24 (k = 4, 64 rows),
+// 3 of 128^2 1.05 / 0.94, 6 of four sizes 3.11 / 2.91.
+constexpr int kParamInstances = 64;
+struct BatchParam {
+    const float *u, *v;
+    float *su, *sv;
+    int nn, nm, bands, rows;
+    unsigned warp_begin;
+    Coef<float> p;
+};
+struct BatchParams {
+    BatchParam d[kParamInstances];
+    int n;
+};
+
+template <int K, int H, int RX, int BC>
+__global__ void __launch_bounds__(kBatchBlock)
+k_batch_param(const __grid_constant__ BatchParams tab, int flip) {
+    static_assert(kTemporalWarps == 1, "a block is one warp of one instance");
+    pdl_wait();
+    const unsigned wid = blockIdx.x;
+    int i = 0;
+#pragma unroll
+    for (int step = kParamInstances / 2; step > 0; step /= 2)
+        if (i + step < tab.n && tab.d[i + step].warp_begin <= wid) i += step;
+    const BatchParam &d = tab.d[i];
+    const int local = (int)(wid - d.warp_begin);
+    const float *su = flip ? d.su : d.u, *sv = flip ? d.sv : d.v;
+    float *du = flip ? const_cast<float *>(d.u) : d.su, *dv = flip ? const_cast<float *>(d.v) : d.sv;
+    temporal_strip<float, K, H, RX, BC>(local % d.bands, local / d.bands, su, sv, du, dv, d.nn, d.nm, d.rows, d.p);
+    pdl_trigger();
+}
+
+template <int K, int H>
+cudaError_t batch_param_launch(int reaction, int boundary, const BatchParams &tab, unsigned nwarps, int flip, cudaStream_t s) {
+    return with_model(reaction, boundary, [&](auto rx, auto bc) {
+        const cudaError_t e = launch_k(k_batch_param<K, H, decltype(rx)::value, decltype(bc)::value>, nwarps, kBatchBlock, 0,
+                                       s, tab, flip);
+        count_launches(1);
+        return e;
+    });
+}
+
 // One depth, every model of the single-grid kernels (T = float, double,
 // __nv_bfloat16 or __half planes; 16-bit planes round once per launch).
 template <typename T, int K, int H>
@@ -73,3 +122,7 @@ cudaError_t batch_launch_khr(int reaction, int boundary, const BatchDesc *tab, i
                                                   cudaStream_t)
 #define RDK_INSTANTIATE_BATCH(TT, KK, HH) template RDK_BATCH_KHR_SIG(TT, KK, HH);
 #define RDK_EXTERN_BATCH(TT, KK, HH) extern template RDK_BATCH_KHR_SIG(TT, KK, HH);
+#define RDK_BATCH_PARAM_SIG(KK, HH) \
+    cudaError_t rdk::batch_param_launch<KK, HH>(int, int, const rdk::BatchParams &, unsigned, int, cudaStream_t)
+#define RDK_INSTANTIATE_BATCH_PARAM(KK, HH) template RDK_BATCH_PARAM_SIG(KK, HH);
+#define RDK_EXTERN_BATCH_PARAM(KK, HH) extern template RDK_BATCH_PARAM_SIG(KK, HH);

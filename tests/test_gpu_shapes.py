@@ -114,3 +114,18 @@ def test_training_results_outlive_later_calls(rd):
                 u.detach().zero_()
         out.append((kept, *torch.autograd.grad(loss, (u0, v0, t))))
     assert all(torch.equal(a, b) for a, b in zip(*out))
+
+
+@pytest.mark.parametrize("n", [1, 2, 63, 64, 65])
+def test_number_of_instances(rd, n):
+    """Both sides of the number of instances whose table travels with the launch."""
+    specs = [{"nn": 5 + i % 7, "nm": 4 * (1 + i % 40), "params": inp.default_params(Du=0.002 * (i + 1))} for i in range(n)]
+    b = rd.Batch(specs, dtype=torch.float32, boundary="zeroflux")
+    xs = [torch.from_numpy(inp.uniform_field(100 + i, s["nn"], s["nm"])).float().cuda() for i, s in enumerate(specs)]
+    for i, x in enumerate(xs):
+        b.set_state(i, x, -x)
+    b.run(11)
+    for i, (s, x) in enumerate(zip(specs, xs)):
+        ref = gpu_run(rd, x.double().cpu().numpy(), -x.double().cpu().numpy(), s["params"], 11, torch.float32, "generic",
+                      boundary="zeroflux")
+        assert all((t.cpu().numpy() == r).all() for t, r in zip(b.state(i), ref)), i

@@ -517,16 +517,27 @@ int default_k_ragged(int64_t nn, int64_t nm) { return model_depth(kRaggedBeats, 
 // 121 / 110.
 bool auto_single_step(int dtype) { return dtype == RDCNN_F64; }
 
-// The single-step kernel is fastest with short strips (more warps in flight);
-// the 16-bit single step (the ring pipeline at depth 1, 8 values per lane)
-// with 32-row strips (measured at 4096^2, bf16: 4 / 8 / 16 / 32 / 64 rows =
-// 507 / 570 / 627 / 672 / 574 Gcell/s).
+// The single-step kernel is fastest with short strips (more warps in flight).
+// The 16-bit single step (the ring pipeline at depth 1, 8 values per lane where
+// rows are such vectors) takes the strips of which an SM gets 8, or 16 where
+// those would be longer than 17 rows, and 32 rows from there on.  bf16, us a
+// step, 32 rows / now: 512^2 7.5 / 2.5, 1024^2 7.6 / 3.4, 2048^2 8.0 / 6.5, 4096 x
+// 1000 10.5 / 6.8, 2900 x 3128 14.8 / 11.4; 4096^2 with 31 / 32 rows 23.9 / 23.5.
 // FP64: one row while that leaves warp slots free, else two (us a step, 1 / 2 /
 // 4 / 8 rows: 64^2 2.3 / 3.6 / 5.6 / 10.2, 256^2 3.6 / 3.7 / 5.9 / 10.5, 512^2
 // 10.4 / 9.1 / 10.0 / 11.1, 2048^2 120 / 110 / 110 / 114).
 int default_rows_step1(int dtype, int64_t nn, int64_t nm) {
     if (dtype == RDCNN_F64) return nn * nm <= (int64_t(1) << 16) ? 1 : 2;
-    return is_16bit(dtype) ? 32 : 2;
+    if (!is_16bit(dtype)) return 2;
+    const int64_t outw = nm % 8 == 0 ? 240 : 120;
+    const int64_t bands = (nm + outw - 1) / outw;
+    int64_t rows = 32;
+    for (int per_sm : {8, 16}) {
+        const int64_t strips = std::max<int64_t>(1, sm_count() * per_sm / bands);
+        rows = (nn + strips - 1) / strips;
+        if (rows <= 17) break;
+    }
+    return rows > 27 ? 32 : (int)std::max<int64_t>(rows, 2);
 }
 
 }  // namespace rdk

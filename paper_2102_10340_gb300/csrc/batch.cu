@@ -102,6 +102,7 @@ void batch_shape_f32(const rdcnn_instance *inst, int n, int k_asked, int rows_as
         }
         ++count.back();
     }
+    const int sms = sm_count();
     double least = 1e300;
     for (int K = k_asked ? k_asked : 4; K <= (k_asked ? k_asked : 8); ++K) {
         const int outw = temporal_out_cols(RDCNN_F32, K);
@@ -110,7 +111,7 @@ void batch_shape_f32(const rdcnn_instance *inst, int n, int k_asked, int rows_as
             int64_t warps = 0;
             for (size_t i = 0; i < kinds; ++i)
                 warps += count[i] * ((sizes[i].second + outw - 1) / outw) * ((sizes[i].first + r - 1) / r);
-            const double t = temporal_us(K, warps, r) / K;
+            const double t = temporal_us(K, warps, r, sms) / K;
             if (t < least) { least = t; *k = K; *rows = r; }
             if (rows_asked) break;
         }

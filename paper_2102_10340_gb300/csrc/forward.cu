@@ -281,7 +281,7 @@ int model_depth(const BeatModel &m, int64_t nn, int64_t nm) {
 
 }  // namespace
 
-double temporal_us(int K, int64_t warps, int64_t rows) { return launch_us(kBeats, K, warps, rows, (int64_t)sm_count() * 8); }
+double temporal_us(int K, int64_t warps, int64_t rows, int sms) { return launch_us(kBeats, K, warps, rows, (int64_t)sms * 8); }
 
 int auto_rows_f32(bool ragged, int K, int64_t nn, int64_t nm) {
     double us;

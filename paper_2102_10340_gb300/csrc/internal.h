@@ -179,8 +179,9 @@ int auto_rows_temporal(int K, int64_t nn, int64_t nm, int bands, int blocks_per_
                        int warps_per_block);
 // The same for FP32 planes with 4 values per lane (launch model in forward.cu).
 int auto_rows_f32(bool ragged, int K, int64_t nn, int64_t nm);
-// us of an FP32 temporal launch of depth K with that many strips of that many rows.
-double temporal_us(int K, int64_t warps, int64_t rows);
+// us of an FP32 temporal launch of depth K with that many strips of that many
+// rows on a device of `sms` SMs.
+double temporal_us(int K, int64_t warps, int64_t rows, int sms);
 // u = v = ka * x; x may alias u.
 cudaError_t launch_init(int dtype, const void *x, void *u, void *v, double ka, int64_t n,
                         cudaStream_t s);

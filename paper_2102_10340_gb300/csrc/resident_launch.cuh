@@ -3,6 +3,8 @@
 // parallel.
 #pragma once
 
+#include <atomic>
+
 #include "internal.h"
 #include "resident.cuh"
 
@@ -13,20 +15,15 @@ constexpr size_t resident_smem(int warps) {  // two parities x two directions x 
     return (size_t)2 * warps * 2 * 2 * 128 * V + (size_t)16 * warps;
 }
 
-// Whether a cluster of `blocks` blocks of `warps` warps can run on this device
-// (more than eight blocks: the non-portable size, which not every partition of
-// a GPU has room for).
+// The most blocks, 16 or 8, of a cluster of the largest blocks that the current
+// device can run (more than eight is the non-portable size, which not every
+// partition of a GPU has room for); 0: none.
 template <int V, int RX, int BC, bool RAG>
-bool resident_runs(int blocks, int warps) {
-    // the most blocks of the largest size that one cluster may have
-    static const int most = [] {
-        auto *k = k_resident<V, RX, BC, RAG>;
-        const int wmax = ResWarps<V>::value;
-        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)resident_smem<V>(wmax)) != cudaSuccess ||
-            cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-            (void)cudaGetLastError();
-            return 0;
-        }
+int resident_most() {
+    auto *k = k_resident<V, RX, BC, RAG>;
+    const int wmax = ResWarps<V>::value;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)resident_smem<V>(wmax)) == cudaSuccess &&
+        cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
         for (int c : {16, 8}) {
             cudaLaunchAttribute at[1];
             at[0].id = cudaLaunchAttributeClusterDimension;
@@ -42,8 +39,22 @@ bool resident_runs(int blocks, int warps) {
             if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) == cudaSuccess && n > 0) return c;
             (void)cudaGetLastError();
         }
-        return 0;
-    }();
+    }
+    (void)cudaGetLastError();
+    return 0;
+}
+
+// Whether a cluster of `blocks` blocks of `warps` warps can run; asked once per device.
+template <int V, int RX, int BC, bool RAG>
+bool resident_runs(int blocks, int warps) {
+    static std::atomic<int> known[16];  // resident_most() + 1 by device
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 16) return false;
+    int most = known[dev].load(std::memory_order_acquire) - 1;
+    if (most < 0) {
+        most = resident_most<V, RX, BC, RAG>();
+        known[dev].store(most + 1, std::memory_order_release);
+    }
     return blocks <= most && warps <= ResWarps<V>::value;
 }
 

@@ -186,10 +186,10 @@ int rdcnn_set_state(rdcnn_t *h, const void *u0, const void *v0, int on_device);
  * otherwise an explicit request returns RDCNN_EINVAL, and AUTO runs F32
  * planes through the temporal pipeline with elements copied one by one, others
  * through GENERIC.  AUTO on F64 planes is STEP1 unless a depth is asked for
- * (k or tune->k).  AUTO on F32 grids of 16 to 256 columns and up to 512 (129
- * columns and more) or 1024 rows, with no k and no tune, advances whole
- * stretches of the run in one launch of one thread-block cluster that holds
- * the state in registers: the same bits.  The handle's reaction and boundary apply to every
+ * (k or tune->k).  AUTO on F32 grids of 16 to 384 columns and up to 1024 (129
+ * columns and more: 512, 257 and more: 256) rows, with no k and no tune,
+ * advances whole stretches of the run in one launch of one thread-block
+ * cluster that holds the state in registers: the same bits.  The handle's reaction and boundary apply to every
  * variant; RDCNN_VARIANT_TEMPORAL2 takes FP32 / FP64 handles only.
  * Errors: RDCNN_ESTATE, RDCNN_EINVAL, RDCNN_ECUDA. */
 int rdcnn_run(rdcnn_t *h, int64_t T, int variant, int k);

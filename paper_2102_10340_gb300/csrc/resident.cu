@@ -7,6 +7,7 @@
 extern template RDK_RESIDENT_SIG(2);
 extern template RDK_RESIDENT_SIG(4);
 extern template RDK_RESIDENT_SIG(8);
+extern template RDK_RESIDENT_SIG(12);
 
 namespace rdk {
 
@@ -27,11 +28,14 @@ struct ResShape {
 // faster over all of its range and at any number of steps (T = 1024, us: 16 x 256
 // 805 -> 345, 64^2 857 -> 181, 1024 x 128 1187 -> 740, 512 x 256 1187 -> 763,
 // 251 x 253 1412 -> 709; T = 2: one launch in the place of one and two copies).
+// 257 to 384 columns (12 a lane) only up to 256 rows: us a step, launches /
+// resident: 64 x 384 0.79 / 0.39, 128 x 300 0.79 / 0.46, 256 x 260 0.80 / 0.68, but
+// 300^2 0.82 / 1.03, 384^2 0.96 / 1.04.
 ResShape resident_shape(int64_t nn, int64_t nm) {
     ResShape s;
-    if (nm < 16 || nm > 256 || nn < 1) return s;
-    const int V = nm <= 64 ? 2 : nm <= 128 ? 4 : 8;
-    const int most = V == 8 ? ResWarps<8>::value : ResWarps<4>::value;
+    if (nm < 16 || nm > (nn <= 256 ? 384 : 256) || nn < 1) return s;
+    const int V = nm <= 64 ? 2 : nm <= 128 ? 4 : nm <= 256 ? 8 : 12;
+    const int most = V >= 8 ? ResWarps<8>::value : ResWarps<4>::value;
     const int blocks = (int)std::min<int64_t>(16, nn);
     const int64_t per_block = (nn + blocks - 1) / blocks;
     const int64_t rows = std::min<int64_t>(kResRows, (per_block + 3) / 4);
@@ -58,6 +62,7 @@ cudaError_t launch_resident(int reaction, int boundary, void *u, void *v, int64_
         case 2: return go(IntC<2>{});
         case 4: return go(IntC<4>{});
         case 8: return go(IntC<8>{});
+        case 12: return go(IntC<12>{});
         default: return cudaErrorNotSupported;
     }
 }

@@ -52,8 +52,9 @@ struct ResArgs {
     Coef<float> p;
 };
 
-// Most warps of a block: V = 8 needs up to 172 registers a thread, V = 4 up to 100.
-template <int V> struct ResWarps : IntC<V == 8 ? 8 : 16> {};
+// Most warps of a block: V = 12 needs up to 255 registers a thread, V = 8 up to
+// 172, V = 4 up to 100.
+template <int V> struct ResWarps : IntC<V >= 8 ? 8 : 16> {};
 
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
@@ -69,7 +70,9 @@ __device__ __forceinline__ unsigned in_cluster(unsigned a, unsigned rank) {
 // it holds the last V columns, the first V - rem of them also held by the lane
 // before it (rem = NM mod V): its west neighbour is that lane's element rem - 1,
 // and that lane's east neighbour is its element V - rem.
-template <int V, int BC, bool RAG> struct Ring {
+// RAG = 1: any width; 4: widths that are multiples of 4, so that rem is one and
+// fewer elements are to choose from (V = 12; with V = 8 it made no difference).
+template <int V, int BC, int RAG> struct Ring {
     int west_src, east_src;
     bool first, end;         // lane holds column 0 / the last column
     bool pw[V], pe[V];       // element handed west -> east / east -> west by this lane
@@ -80,16 +83,16 @@ template <int V, int BC, bool RAG> struct Ring {
         east_src = lane >= last ? 0 : lane + 1;
 #pragma unroll
         for (int k = 0; k < V; ++k) {
-            pw[k] = RAG && lane == last - 1 && k == rem - 1;
-            pe[k] = RAG && end && k == V - rem;
+            pw[k] = RAG > 0 && lane == last - 1 && k == rem - 1;
+            pe[k] = RAG > 0 && end && k == V - rem;
         }
     }
     // Element -1 of a row held as a[0 .. V-1] by the lanes.
     __device__ __forceinline__ float west(const float (&a)[V]) const {
         float x = a[V - 1];
-        if constexpr (RAG) {
+        if constexpr (RAG > 0) {
 #pragma unroll
-            for (int k = 0; k < V - 1; ++k) x = pw[k] ? a[k] : x;
+            for (int k = RAG - 1; k < V - 1; k += RAG) x = pw[k] ? a[k] : x;
         }
         x = __shfl_sync(kFull, x, west_src);
         return (BC == BC_MIRROR && first) ? a[0] : x;
@@ -97,9 +100,9 @@ template <int V, int BC, bool RAG> struct Ring {
     // Element V.
     __device__ __forceinline__ float east(const float (&a)[V]) const {
         float x = a[0];
-        if constexpr (RAG) {
+        if constexpr (RAG > 0) {
 #pragma unroll
-            for (int k = 1; k < V; ++k) x = pe[k] ? a[k] : x;
+            for (int k = RAG; k < V; k += RAG) x = pe[k] ? a[k] : x;
         }
         x = __shfl_sync(kFull, x, east_src);
         return (BC == BC_MIRROR && end) ? a[V - 1] : x;
@@ -296,14 +299,14 @@ template <int V, int NR, int BC> struct RowSums {
 
 // The whole run of a warp that holds NR rows from row r0 on; w = its index in
 // the block, g = in the cluster.
-template <int V, int NR, int RX, int BC, bool RAG>
+template <int V, int NR, int RX, int BC, int RAG>
 __device__ __forceinline__ void resident_rows(const ResArgs &a, int r0, int w, int g, unsigned rank, unsigned smem) {
     constexpr bool OUT = (RX == RX_CENN);   // sums over the outputs clamp1(u); v is constant
     constexpr int F = OUT ? 1 : 2;          // handed fields
     const int lane = threadIdx.x & 31;
     const int last = (a.nm - 1) / V;
     const Ring<V, BC, RAG> ring(lane, last, a.nm % V);
-    const int col = RAG && lane == last ? a.nm - V : lane * V;
+    const int col = RAG > 0 && lane == last ? a.nm - V : lane * V;
     const bool in_use = lane <= last;
 
     float U[NR][V], W[NR][V];
@@ -338,7 +341,7 @@ __device__ __forceinline__ void resident_rows(const ResArgs &a, int r0, int w, i
     if (down_far) down_to = in_cluster(down_to, down_rank), down_bar = in_cluster(down_bar, down_rank);
     const unsigned from = slot(w, 0, lane);
     // element V of the handed row above, where its lane stored it
-    const int east_e = RAG && lane == last - 1 ? V - a.nm % V : 0;
+    const int east_e = RAG > 0 && lane == last - 1 ? V - a.nm % V : 0;
     const unsigned from_east = slot(w, 0, ring.east_src) + (east_e / 4) * 512 + (east_e % 4) * 4;
     // bytes from the neighbours in other blocks
     const unsigned bytes = ((int)(up_far && !top) + (int)(down_far && !bottom)) * F * kSlot;
@@ -447,7 +450,7 @@ __device__ __forceinline__ void resident_rows(const ResArgs &a, int r0, int w, i
 }
 
 // One cluster; warp g of it holds rows g NN / nwarps .. (g + 1) NN / nwarps - 1.
-template <int V, int RX, int BC, bool RAG>
+template <int V, int RX, int BC, int RAG>
 __global__ void __launch_bounds__(32 * ResWarps<V>::value, 1)
 k_resident(const ResArgs a) {
     extern __shared__ __align__(16) unsigned char res_smem[];

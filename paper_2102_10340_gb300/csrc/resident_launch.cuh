@@ -18,7 +18,7 @@ constexpr size_t resident_smem(int warps) {  // two parities x two directions x 
 // The most blocks, 16 or 8, of a cluster of the largest blocks that the current
 // device can run (more than eight is the non-portable size, which not every
 // partition of a GPU has room for); 0: none.
-template <int V, int RX, int BC, bool RAG>
+template <int V, int RX, int BC, int RAG>
 int resident_most() {
     auto *k = k_resident<V, RX, BC, RAG>;
     const int wmax = ResWarps<V>::value;
@@ -45,7 +45,7 @@ int resident_most() {
 }
 
 // Whether a cluster of `blocks` blocks of `warps` warps can run; asked once per device.
-template <int V, int RX, int BC, bool RAG>
+template <int V, int RX, int BC, int RAG>
 bool resident_runs(int blocks, int warps) {
     static std::atomic<int> known[16];  // resident_most() + 1 by device
     int dev = 0;
@@ -67,7 +67,7 @@ cudaError_t resident_launch_v(int reaction, int boundary, void *u, void *v, int6
         constexpr int RX = decltype(rx)::value;
         constexpr int BC = decltype(bc)::value;
         auto launch = [&](auto rag) -> cudaError_t {
-            constexpr bool RAG = decltype(rag)::value != 0;
+            constexpr int RAG = decltype(rag)::value;
             if (!resident_runs<V, RX, BC, RAG>(blocks, warps)) return cudaErrorNotSupported;
             cudaLaunchAttribute at[2];
             at[0].id = cudaLaunchAttributeClusterDimension;
@@ -86,7 +86,11 @@ cudaError_t resident_launch_v(int reaction, int boundary, void *u, void *v, int6
             count_launches(1);
             return e != cudaSuccess ? e : cudaGetLastError();
         };
-        return nm % V == 0 ? launch(IntC<0>{}) : launch(IntC<1>{});
+        if (nm % V == 0) return launch(IntC<0>{});
+        if constexpr (V > 8) {
+            if (nm % 4 == 0) return launch(IntC<4>{});
+        }
+        return launch(IntC<1>{});
     });
 }
 

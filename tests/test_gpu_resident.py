@@ -1,6 +1,6 @@
-"""AUTO on FP32 grids up to 256 columns wide (one cluster holds the state, one launch a stretch of
-steps) against the one-thread-per-cell kernel: the same bits, at the edges of every lane width (2, 4
-and 8 columns a lane, with a last lane that overlaps the one before it), with 1 to 4 rows a warp, one
+"""AUTO on FP32 grids up to 384 columns wide (one cluster holds the state, one launch a stretch of
+steps) against the one-thread-per-cell kernel: the same bits, at the edges of every lane width (2, 4,
+8 and 12 columns a lane, with a last lane that overlaps the one before it), with 1 to 4 rows a warp, one
 to sixteen blocks, and on both sides of the range's ends."""
 import pytest
 import torch
@@ -12,7 +12,8 @@ pytestmark = pytest.mark.gpu
 
 SHAPES = [(1, 16), (1, 64), (2, 17), (5, 96), (15, 15), (16, 16), (17, 63), (31, 65), (33, 33), (40, 200), (61, 130),
           (64, 64), (100, 128), (129, 127), (200, 250), (255, 251), (256, 256), (260, 255), (512, 256), (513, 256),
-          (1023, 49), (1024, 100), (1025, 64), (48, 257)]
+          (1023, 49), (1024, 100), (1025, 64), (1, 257), (17, 268), (48, 257),
+          (90, 383), (64, 384), (256, 260), (256, 384), (257, 300), (40, 385)]
 MODELS = [("periodic", "fhn"), ("zeroflux", "fhn"), ("periodic", "cenn"), ("zeroflux", "cenn"), ("zeroflux", "none")]
 
 

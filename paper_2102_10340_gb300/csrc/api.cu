@@ -340,7 +340,7 @@ int run_core(rdcnn_t *h, int64_t T, int variant, int k, int64_t every, MarkFn ma
     if (rv < 0) return rv;
     // FP32 planes that are not vector-aligned: depth does not change their
     // bits, so AUTO steps them K at a time too (1003 x 1021, 100 steps: 758 ->
-    // 272 us).  16-bit planes round once per launch and stay with one step a
+    // 224 us).  16-bit planes round once per launch and stay with one step a
     // launch; FP64 planes are fastest with one (auto_single_step).  A depth that
     // only the vectorised variants would reject is ignored here, as GENERIC
     // ignores it.

@@ -129,3 +129,20 @@ def test_number_of_instances(rd, n):
         ref = gpu_run(rd, x.double().cpu().numpy(), -x.double().cpu().numpy(), s["params"], 11, torch.float32, "generic",
                       boundary="zeroflux")
         assert all((t.cpu().numpy() == r).all() for t, r in zip(b.state(i), ref)), i
+
+
+def test_captured_states_and_odd_runs(rd):
+    """Setting a state and a run that ends in the scratch planes, recorded into the caller's graph."""
+    nn, nm = 40, 300
+    x, y = (torch.from_numpy(inp.uniform_field(s, nn, nm)).float().cuda() for s in (83, 84))
+    g, h = (rd.Grid(nn, nm, inp.default_params()) for _ in range(2))
+    for t in (g, h):
+        t.set_state(x, y).run(3, variant="step1")
+    graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.graph(graph, stream=side):
+        g.set_state(y, x).run(5, variant="step1")
+    h.set_state(y, x).run(5, variant="step1")
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(g.u, h.u) and torch.equal(g.v, h.v)

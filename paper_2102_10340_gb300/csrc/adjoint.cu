@@ -80,7 +80,7 @@ k_reduce_partials(const double *__restrict__ partial, int n, double dt, double *
 // GPU, so it computes no cell twice, unlike the pipeline (k_adjoint_pipe), and
 // its warps are short: on a small grid the pipeline's few strips leave most SMs
 // idle.  us a step of the reverse sweep, pipeline with k = 2 / this: 64^2 11.1 /
-// 5.8, 128^2 11.2 / 6.4, 256^2 16.9 / 9.8, 512^2 31.7 / 24.7, 1024^2 101 / 78.
+// 5.4, 128^2 11.2 / 5.4, 256^2 16.9 / 9.3, 512^2 31.7 / 24.1, 1024^2 101 / 77.
 // Sums: each lane's six, added over groups of four lanes and then to the
 // group's record in `partial` (one record per 4 lanes of every warp, read and
 // written by the same lane at each launch), so no launch reduces a whole warp.
@@ -106,6 +106,14 @@ k_adjoint_step(const double *__restrict__ lu, const double *__restrict__ lv, dou
     const bool edge_e = active && (lane == 31 || col + V >= nm);
     const int r0 = wid / bands * rows, r1 = min(r0 + rows, nn);
     double rg[6] = {0, 0, 0, 0, 0, 0};
+    // the group's record, read ahead of the rows: read where it is added to, its
+    // latency came on top of theirs (128^2 6.4 us a step)
+    double2 *rec = reinterpret_cast<double2 *>(partial + ((int64_t)wid * kRevRecords + lane / 4) * 6);
+    double2 old[3];
+    if ((lane & 3) == 0) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q) old[q] = rec[q];
+    }
     for (int r = r0; r < r1; ++r) {
         const int64_t rn = r == 0 ? (zf ? 0 : nn - 1) : r - 1, rs = r + 1 == nn ? (zf ? r : 0) : r + 1;
         const int64_t at = (int64_t)r * nm + col;
@@ -141,9 +149,9 @@ k_adjoint_step(const double *__restrict__ lu, const double *__restrict__ lv, dou
         rg[q] = add_rn(rg[q], __shfl_xor_sync(kFull, rg[q], 2));
     }
     if ((lane & 3) == 0) {
-        double *rec = partial + ((int64_t)wid * kRevRecords + lane / 4) * 6;
 #pragma unroll
-        for (int q = 0; q < 6; ++q) rec[q] = add_rn(rec[q], rg[q]);
+        for (int q = 0; q < 3; ++q)
+            rec[q] = make_double2(add_rn(old[q].x, rg[2 * q]), add_rn(old[q].y, rg[2 * q + 1]));
     }
     pdl_trigger();
 }
@@ -155,7 +163,7 @@ struct StepShape {
 
 // Rows per warp: one up to 2^18 cells, four above, where the sums' additions (18
 // of 68 FP64 instructions of a one-row warp) weigh more.  us a step of the whole
-// reverse sweep, rebuilds included, with 1 / 2 / 4 / 8 rows: 128^2 6.4 / 8.1 / 11.4
+// reverse sweep, rebuilds included, with 1 / 2 / 4 / 8 rows (records read last): 128^2 6.4 / 8.1 / 11.4
 // / 18.8, 512^2 24.7 / 24.9 / 27.8 / 31.9, 1024^2 91.6 / 82.8 / 77.8 / 78.8.
 StepShape step_shape(int64_t nn, int64_t nm) {
     StepShape q;

@@ -40,6 +40,17 @@
  * the batched sweep (rdcnn_batch_run*, rdcnn_batch_summary); the adjoint,
  * static-scratch and TEMPORAL2 paths return RDCNN_EINVAL.
  *
+ * Rounding: all variants form a cell alike, so they give the same bits (16-bit
+ * planes: at the same steps per launch).  FP64 grids, and zero-flux grids of
+ * every type, add the four neighbours as (north + south) + (west + east),
+ * which a reflection of the rows or columns leaves unchanged: a
+ * mirror-symmetric state stays mirror-symmetric bit for bit.  FP32 and 16-bit
+ * grids on the torus add them as (north + west) + (south + east), unchanged by
+ * transposition and by half a turn only: mirror symmetry holds up to rounding,
+ * which grows where the model magnifies it (512^2, FP32, random symmetric
+ * start, default gene: cells differ by up to 2e-5 after 100 steps, 3e-4 after
+ * 200).
+ *
  * Conventions shared by every entry point
  *  - Layout: one plane per field, row-major [NN][NM], element (i, j) at
  *    offset i * NM + j; i is the row (NN rows), j the column (NM columns).

@@ -246,16 +246,22 @@ __device__ __forceinline__ float clamp1(float x) { return fminf(fmaxf(x, -1.0f),
 __device__ __forceinline__ double clamp1(double x) { return fmin(fmax(x, -1.0), 1.0); }
 
 // Sum of the four neighbours of a cell (rows i-1 / i+1, columns j-1 / j+1).
-// On the torus the sum is grouped (n + w) + (s + e): s + e of cell (i, j) is
-// n + w of cell (i+1, j+1), so the pipelines of temporal.cuh form each pair
-// once and spend two additions per cell instead of three, with these bits.
+// FP32 arithmetic on the torus groups the sum (n + w) + (s + e): s + e of cell
+// (i, j) is n + w of cell (i+1, j+1), so the pipelines of temporal.cuh form each
+// pair once and spend two additions per cell instead of three, with these bits.
+// This grouping is unchanged by transposition and by half a turn, but not by a
+// reflection: a mirror-symmetric FP32 start stays so up to rounding only.
 // Under zero flux the grouping is (n + s) + (w + e), which a reflection about
 // a row or a column leaves unchanged (IEEE addition commutes), as the mirrored
-// halos need.
+// halos need; and so it is in FP64 on the torus, whose kernels share no pairs
+// (StageRows::kPair): a mirror-symmetric start stays so bit for bit.
+template <int BC, typename T> struct PairSums {
+    static constexpr bool value = BC == BC_WRAP && std::is_same<T, float>::value;
+};
 template <int BC, typename T>
 __device__ __forceinline__ T nbr_sum(T n, T s, T w, T e) {
-    if constexpr (BC == BC_MIRROR) return add_rn(add_rn(n, s), add_rn(w, e));
-    else return add_rn(add_rn(n, w), add_rn(s, e));
+    if constexpr (PairSums<BC, T>::value) return add_rn(add_rn(n, w), add_rn(s, e));
+    else return add_rn(add_rn(n, s), add_rn(w, e));
 }
 
 // One cell from its centre and its neighbour sums su, sv.

@@ -512,9 +512,9 @@ int default_k_ragged(int64_t nn, int64_t nm) { return model_depth(kRaggedBeats, 
 // FP64 runs at 1/64 of the FP32 rate, so the FP64 pipe bounds every grid that
 // fills the GPU, and a halo cell costs as much as an owned one: the single
 // step, which computes no cell twice, beats every depth at every size.  us a
-// step (k = 4 / best depth / single step): 64^2 6.5 / 3.6 / 2.3, 256^2 6.5 /
-// 4.7 / 3.6, 512^2 16.6 / 9.8 / 9.1, 1024^2 37.1 / 33.0 / 29.6, 2048^2 135 /
-// 121 / 110.
+// step (k = 4 / best depth / single step): 64^2 7.3 / 5.9 / 2.3, 256^2 7.4 /
+// 5.9 / 3.5, 512^2 18.7 / 10.9 / 9.3, 1024^2 42.4 / 37.4 / 30.6, 2048^2 156 /
+// 136 / 113.
 bool auto_single_step(int dtype) { return dtype == RDCNN_F64; }
 
 // The single-step kernel is fastest with short strips (more warps in flight).

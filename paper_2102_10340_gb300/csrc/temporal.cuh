@@ -197,17 +197,17 @@ template <int BC> struct RowWalk {
 // The rows one stage keeps between beats, and the neighbour sums they give.
 // cen = row q of the stage's input, C = row q + 1, just arrived.
 //
-// Torus, linear sums: the cell sum is (n + w) + (s + e), and s + e of cell
+// FP32 torus, linear sums: the cell sum is (n + w) + (s + e), and s + e of cell
 // (q, j) is n + w of cell (q + 1, j + 1).  So a stage keeps row q and the
 // pair sums acc(j) = row_{q-1}(j+1) + row_q(j) instead of rows q - 1 and q:
 // the sum of a cell is its own new pair (row_q(j+1) + C(j)) plus the old pair
 // one column to the west -- two additions per field instead of three, at the
 // same registers and the same two shuffles.  4096^2, K = 8:
 // 92.7 -> 82.7 us a launch.
-// Zero flux: rows q - 1 and q, three additions (nbr_sum says why).
+// Zero flux and FP64: rows q - 1 and q, three additions (nbr_sum says why).
 // CeNN cell (OUT): the sums run over the outputs y = clamp(x), clamped once
-// when a row arrives and kept (pair sums and y of row q on the torus, y of
-// rows q - 1 and q under zero flux) instead of once per neighbour; v is
+// when a row arrives and kept (pair sums and y of row q on the FP32 torus, y of
+// rows q - 1 and q otherwise) instead of once per neighbour; v is
 // constant, so it needs no sums.  4096^2, K = 8: torus 73.5 -> 57.2 us a
 // launch, zero flux 75.7 -> 69.6 us.
 //
@@ -216,7 +216,7 @@ template <int BC> struct RowWalk {
 // three-phase ones hold rows q - 1, q, q + 1 in row[PH], row[PH + 1],
 // row[PH + 2].
 template <typename T, int V, int K, int BC, bool OUT> struct StageRows {
-    static constexpr bool kPair = (BC == BC_WRAP && K > 1);
+    static constexpr bool kPair = PairSums<BC, T>::value && K > 1;
     static constexpr int kPhases = (!kPair && !OUT) ? 3 : 2;
     Slice<T, V> row[kPhases];
     T acc[2][V];

@@ -236,7 +236,9 @@ int rdcnn_get_state(rdcnn_t *h, void *u_out, void *v_out, int to_device);
  * Snapshot s (s = 0 .. T/every, integer division) is the state after
  * s * every steps, written to u_snap + s*NN*NM and v_snap + s*NN*NM
  * (elements of the handle's dtype).  snap_on_device = 1: device arrays,
- * copied on the bound stream, asynchronous.  snap_on_device = 0: host arrays
+ * written on the bound stream, asynchronous; the bound planes may be slots of
+ * them, and one array may take both fields (it then holds v).  snap_on_device
+ * = 0: host arrays
  * (pinned memory lets the copies overlap the steps); each snapshot passes
  * through a device staging slot of 2 planes taken from `staging`
  * (staging_bytes / (2 * plane bytes) slots, at least one) and is copied on a

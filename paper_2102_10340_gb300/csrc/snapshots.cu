@@ -6,8 +6,9 @@
 // Launches are cut so that one ends exactly at every multiple of `every`;
 // after it, the state planes are copied
 //  - to device snapshots: the launch that ends there writes the caller's array
-//    itself, and the next one reads it (copied where it is not aligned, or
-//    where one launch holds the whole grid, resident.cuh);
+//    itself, and the next one reads it (copied where it is not aligned or
+//    overlaps other planes, or where one launch holds the whole grid,
+//    resident.cuh);
 //  - to host snapshots: into a caller-provided device staging slot on the
 //    compute stream, then to the host on a second stream (created once per
 //    handle), so that the transfer overlaps the following steps.  A staging
@@ -61,9 +62,29 @@ int on_mark(void *ctx, int64_t t, const void *cu, const void *cv) {
     return take_snapshot(c, t / c.every, cu, cv);
 }
 
+// Whether the steps may write device snapshots themselves: `slots` slots in memory of
+// this device that share no byte with one another's array, the bound planes or the
+// workspace.  A launch reads one pair of planes while it writes another, and the
+// next one reads the slots; copies may overlap them (state planes that are
+// slots of the arrays, one array for both fields).
+bool slots_stand_alone(const SnapCtx &c, int64_t slots) {
+    struct Span { const char *p; size_t n; };
+    const rdcnn_t *h = c.h;
+    const Span s[] = {{c.u_snap, (size_t)slots * c.plane},
+                      {c.v_snap, (size_t)slots * c.plane},
+                      {(const char *)h->u, c.plane},
+                      {(const char *)h->v, c.plane},
+                      {(const char *)h->ws, plane_stride(c.plane) + c.plane}};
+    for (int i = 0; i < 2; ++i)
+        for (int j = i + 1; j < 5; ++j)
+            if (s[i].p < s[j].p + s[j].n && s[j].p < s[i].p + s[i].n) return false;
+    return on_this_device(c.u_snap) && on_this_device(c.v_snap);
+}
+
 // Device snapshots: the launch that completes the step writes the slot (768 x
 // 1024, every 20 of 200 steps: 493 -> 420 us against a pair of copies per slot).  Slots
-// off the vectorised kernels' alignment, and arrays on another device, are copied to.
+// off the vectorised kernels' alignment, on another device or overlapping other
+// planes are copied to.
 bool snapshot_planes(void *ctx, int64_t t, void **du, void **dv) {
     SnapCtx &c = *static_cast<SnapCtx *>(ctx);
     if (!c.direct) return false;
@@ -93,7 +114,7 @@ int rdcnn_run_snapshots(rdcnn_t *h, int64_t T, int64_t every, void *u_snap, void
     c.u_snap = (char *)u_snap;
     c.v_snap = (char *)v_snap;
     c.on_device = snap_on_device != 0;
-    c.direct = c.on_device && on_this_device(u_snap) && on_this_device(v_snap);
+    c.direct = c.on_device && slots_stand_alone(c, T / every + 1);
     if (!c.on_device) {
         c.staging = (char *)staging;
         c.n_stage = staging ? (int)std::min<size_t>(staging_bytes / (2 * c.plane), 1 << 16) : 0;

@@ -200,7 +200,9 @@ int rdcnn_set_state(rdcnn_t *h, const void *u0, const void *v0, int on_device);
  * (k or tune->k).  AUTO on F32 grids of 16 to 384 columns and up to 1024 (129
  * columns and more: 512, 257 and more: 256) rows, with no k and no tune,
  * advances whole stretches of the run in one launch of one thread-block
- * cluster that holds the state in registers: the same bits.  The handle's reaction and boundary apply to every
+ * cluster that holds the state in registers: the same bits (or, should its
+ * blocks wait for one another for more than ten seconds, NaN in every cell of
+ * u and v).  The handle's reaction and boundary apply to every
  * variant; RDCNN_VARIANT_TEMPORAL2 takes FP32 / FP64 handles only.
  * Errors: RDCNN_ESTATE, RDCNN_EINVAL, RDCNN_ECUDA. */
 int rdcnn_run(rdcnn_t *h, int64_t T, int variant, int k);
@@ -223,6 +225,16 @@ int rdcnn_run(rdcnn_t *h, int64_t T, int variant, int k);
  * TEMPORAL: the variants that a caller may ask for by name.  Queries the current device's SM count and kernel
  * occupancy.  Errors: RDCNN_EINVAL (as rdcnn_run would return). */
 int rdcnn_plan(const rdcnn_t *h, int *variant, rdcnn_tune *out);
+
+/* T steps of Eq. 1 by the one-cluster launches that AUTO takes for small FP32
+ * grids (at most 8192 steps each), whether or not AUTO would take them here:
+ * for tests and measurements.  The blocks of the cluster wait for one
+ * another's rows.  A wait that takes longer than ten seconds gives up; the
+ * launch then ends, and every cell of u and v is NaN.  give_up = 1 shows
+ * that: the kernel waits for an arrival that nobody makes, for a millisecond.
+ * Errors: RDCNN_EINVAL (the grid's size or dtype does not fit a cluster, or
+ * the device has no room for one), RDCNN_ESTATE, RDCNN_ECUDA. */
+int rdcnn_run_cluster(rdcnn_t *h, int64_t T, int give_up);
 
 /* Copy the current state out (the "lastA, lastB" the paper's display
  * function returns, Sec. II.A).  to_device = 0: host buffers, the call

@@ -69,6 +69,7 @@ SIGNATURES = [
     ("rdcnn_init", c_int, [c_vp, c_vp, c_double, c_int]),
     ("rdcnn_set_state", c_int, [c_vp, c_vp, c_vp, c_int]),
     ("rdcnn_run", c_int, [c_vp, c_i64, c_int, c_int]),
+    ("rdcnn_run_cluster", c_int, [c_vp, c_i64, c_int]),
     ("rdcnn_plan", c_int, [c_vp, ctypes.POINTER(c_int), ctypes.POINTER(Tune)]),
     ("rdcnn_get_state", c_int, [c_vp, c_vp, c_vp, c_int]),
     ("rdcnn_run_snapshots", c_int, [c_vp, c_i64, c_i64, c_vp, c_vp, c_int, c_vp, c_size]),

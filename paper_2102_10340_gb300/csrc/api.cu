@@ -321,9 +321,6 @@ static bool ensure_graph(rdcnn_t *h, int variant, int k, void *su, void *sv) {
     return true;
 }
 
-// Most steps of one resident launch: 1 .. 7 ms.
-constexpr int64_t kResidentSteps = 8192;
-
 int run_core(rdcnn_t *h, int64_t T, int variant, int k, int64_t every, MarkFn mark, void *ctx, DestFn dest) {
     if (!h) return set_error(RDCNN_EINVAL, "handle is NULL");
     if (!h->bound) return set_error(RDCNN_ESTATE, "handle is not bound");
@@ -436,6 +433,22 @@ int run_core(rdcnn_t *h, int64_t T, int variant, int k, int64_t every, MarkFn ma
 extern "C" {
 
 int rdcnn_run(rdcnn_t *h, int64_t T, int variant, int k) { return run_core(h, T, variant, k, 0, nullptr, nullptr); }
+
+int rdcnn_run_cluster(rdcnn_t *h, int64_t T, int give_up) {
+    if (!h) return set_error(RDCNN_EINVAL, "handle is NULL");
+    if (!h->bound) return set_error(RDCNN_ESTATE, "handle is not bound");
+    if (T < 0) return set_error(RDCNN_EINVAL, "T must be >= 0");
+    if (h->dtype != RDCNN_F32 || !resident_fits(h->nn, h->nm))
+        return set_error(RDCNN_EINVAL, "a %lld x %lld grid of this dtype does not fit one cluster", (long long)h->nn,
+                         (long long)h->nm);
+    for (int64_t left = T; left > 0; left -= std::min(left, kResidentSteps)) {
+        const cudaError_t e = launch_resident(h->reaction, h->boundary, h->u, h->v, h->nn, h->nm, h->p,
+                                              std::min(left, kResidentSteps), h->stream, give_up != 0);
+        if (e == cudaErrorNotSupported) return set_error(RDCNN_EINVAL, "this device has no room for the cluster");
+        if (e != cudaSuccess) return cuda_error(e, "resident kernel launch");
+    }
+    return RDCNN_OK;
+}
 
 int rdcnn_plan(const rdcnn_t *h, int *variant, rdcnn_tune *out) {
     if (!h || !variant || !out) return set_error(RDCNN_EINVAL, "NULL argument");

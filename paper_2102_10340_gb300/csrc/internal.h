@@ -153,10 +153,13 @@ cudaError_t launch_temporal_split(int dtype, int reaction, int boundary, int k, 
 // Whether a run of an FP32 grid can stay in the registers of one cluster
 // (resident.cuh), and such a run: `steps` steps of (u, v) in place by one
 // launch, or cudaErrorNotSupported, with nothing launched, where this device
-// has no room for the cluster.
+// has no room for the cluster.  The kernel's waits give up after ten seconds,
+// and the state is then NaN in every cell; give_up: they all run out, after a
+// millisecond.
+constexpr int64_t kResidentSteps = 8192;  // most steps of one launch: 1 .. 7 ms
 bool resident_fits(int64_t nn, int64_t nm);
 cudaError_t launch_resident(int reaction, int boundary, void *u, void *v, int64_t nn, int64_t nm,
-                            const rdcnn_params &p, int64_t steps, cudaStream_t s);
+                            const rdcnn_params &p, int64_t steps, cudaStream_t s, bool give_up = false);
 cudaError_t launch_generic(int dtype, int reaction, int boundary, const void *u, const void *v,
                            void *un, void *vn, int64_t nn, int64_t nm, const rdcnn_params &p,
                            cudaStream_t s);

@@ -53,10 +53,11 @@ ResShape resident_shape(int64_t nn, int64_t nm) {
 bool resident_fits(int64_t nn, int64_t nm) { return resident_shape(nn, nm).V != 0; }
 
 cudaError_t launch_resident(int reaction, int boundary, void *u, void *v, int64_t nn, int64_t nm,
-                            const rdcnn_params &p, int64_t steps, cudaStream_t s) {
+                            const rdcnn_params &p, int64_t steps, cudaStream_t s, bool give_up) {
     const ResShape q = resident_shape(nn, nm);
     auto go = [&](auto vv) {
-        return resident_launch_v<decltype(vv)::value>(reaction, boundary, u, v, nn, nm, p, q.blocks, q.warps, steps, s);
+        return resident_launch_v<decltype(vv)::value>(reaction, boundary, u, v, nn, nm, p, q.blocks, q.warps, steps,
+                                                  give_up, s);
     };
     switch (q.V) {
         case 2: return go(IntC<2>{});

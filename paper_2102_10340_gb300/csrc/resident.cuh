@@ -31,10 +31,16 @@
 // step t is over.  Each row handed on is waited for by its receiver, and the
 // blocks leave together, so none is written after its block has left.
 //
+// Waits are bounded.  A warp whose wait gives up sets a flag in every block and
+// ends (give_up): it hands on no more rows, so its neighbours' waits give up in
+// turn.  The flag is read after the barrier that ends the steps, and every warp
+// of the cluster then stores NaNs in both planes: a failed run has no cell that
+// looks like a result.
+//
 // Bound: latency of the hand-over up to 128^2 (64^2: 370 cycles a step, of which
 // about 100 are the sums and the update), one warp's issue rate per scheduler of
-// 16 SMs at 256^2.  us a step, launches -> resident: 64^2 0.84 -> 0.18, 128^2 0.82
-// -> 0.24, 256^2 0.86 -> 0.48.  Measured on the way, 64^2 / 128^2 / 256^2: one
+// 16 SMs at 256^2.  us a step, launches -> resident: 64^2 0.84 -> 0.17, 128^2 0.82
+// -> 0.23, 256^2 0.86 -> 0.44.  Measured on the way, 64^2 / 128^2 / 256^2: one
 // cluster barrier a step 0.34 / 0.46 / 0.68; every row by asynchronous stores
 // 0.26 / 0.38 / 0.74; two rows handed on every second step, with the redundant
 // rows computed, 0.21 / 0.29 / 0.71.
@@ -50,10 +56,12 @@ struct ResArgs {
     float *u, *v;  // state planes, in place
     int nn, nm, steps, blocks, warps;  // blocks of the cluster, warps of a block
     Coef<float> p;
+    uint64_t wait_ns;  // limit of a wait
+    int never;         // arrivals that no warp makes: 1 has every wait give up (for tests)
 };
 
 // Most warps of a block: V = 12 needs up to 255 registers a thread, V = 8 up to
-// 172, V = 4 up to 100.
+// 208, V = 4 up to 126, V = 2 up to 96.
 template <int V> struct ResWarps : IntC<V >= 8 ? 8 : 16> {};
 
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
@@ -172,19 +180,57 @@ __device__ __forceinline__ uint64_t clock_ns() {
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
 }
-// False when the phase has not completed for kResWaitNs: the blocks of a cluster
-// run at the same time, so only a fault of this file could do that.  The warp
-// then waits no more and stores NaNs for its u.
+// False when the phase has not completed for `limit` ns.  The blocks of a cluster
+// run at the same time, so with the usual limit only a fault of this file could
+// do that.
 constexpr uint64_t kResWaitNs = 10ull * 1000 * 1000 * 1000;
-__device__ __forceinline__ bool bar_wait(unsigned bar, unsigned parity) {  // the whole warp, with one answer
+constexpr uint64_t kResGiveUpNs = 1000 * 1000;  // where the wait is meant to run out
+__device__ __forceinline__ bool bar_wait(unsigned bar, unsigned parity, uint64_t limit) {  // the whole warp, with one answer
     bool ok = bar_try(bar, parity);
     if (__all_sync(kFull, ok)) return true;
     const uint64_t t0 = clock_ns();
     for (;;) {
         ok = ok || bar_try(bar, parity);
         if (__all_sync(kFull, ok)) return true;
-        if (__any_sync(kFull, clock_ns() - t0 > kResWaitNs)) return false;
+        if (__any_sync(kFull, clock_ns() - t0 > limit)) return false;
     }
+}
+// The cluster's failure flag: a word behind the mbarriers of each block.
+constexpr uint64_t kResDrainNs = 1000 * 1000;  // an asynchronous store takes about a microsecond
+__device__ __forceinline__ void flag_set(unsigned flag, unsigned rank) {  // block `rank`'s
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(in_cluster(flag, rank)), "r"(1u) : "memory");
+}
+__device__ __forceinline__ bool flag_get(unsigned flag) {
+    unsigned x;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(x) : "r"(flag) : "memory");
+    return x != 0;
+}
+// Rows that nobody waited for may still be on their way: no block leaves before they are in.
+__device__ __forceinline__ void drain() {
+    const uint64_t t0 = clock_ns();
+    while (!__any_sync(kFull, clock_ns() - t0 >= kResDrainNs)) {}
+    cluster_arrive();
+    cluster_wait();
+}
+// The end of a warp (rows r0 .. r0 + nr - 1) whose wait gave up: the barriers that
+// the others pass after their last step, and the thread's exit.  The exit has a
+// predicate (always true: a cluster has blocks), so that the compiler sees no way
+// out of the step loop here; with one, it builds the loop otherwise: us a step at
+// 64^2 / 128^2 / 256^2, a flag and a break 0.196 / 0.265 / 0.476, an exit known as
+// such 0.188 / 0.255 / 0.508, this 0.165 / 0.231 / 0.441 (with the stores unrolled
+// 0.168 / 0.231 / 0.498).
+__device__ __forceinline__ void give_up(const ResArgs &a, int r0, int nr, unsigned flag) {
+    const int lane = threadIdx.x & 31;
+    if (lane < a.blocks) flag_set(flag, lane);
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();
+#pragma unroll 1
+    for (int i = lane; i < nr * a.nm; i += 32)
+        a.u[(int64_t)r0 * a.nm + i] = a.v[(int64_t)r0 * a.nm + i] = __int_as_float(0x7fffffff);
+    __syncwarp();
+    drain();
+    asm volatile("{\n.reg .pred q;\nsetp.ne.u32 q, %0, 0;\n@q exit;\n}" ::"r"(a.blocks) : "memory");
 }
 template <int V>
 __device__ __forceinline__ void hand_load(unsigned a, float (&x)[V]) {
@@ -331,7 +377,7 @@ __device__ __forceinline__ void resident_rows(const ResArgs &a, int r0, int w, i
     const bool top = (BC == BC_MIRROR) && g == 0, bottom = (BC == BC_MIRROR) && g == nwarps - 1;
     // where the first / last row and their arrivals go (parity 0)
     const unsigned bars = smem + 2 * buf_step;  // [warp][parity]
-    const unsigned bar = bars + 16 * w;
+    const unsigned bar = bars + 16 * w, flag = bars + 16 * a.warps;
     const int up_w = w == 0 ? a.warps - 1 : w - 1, down_w = w == a.warps - 1 ? 0 : w + 1;
     const unsigned up_rank = rank == 0 ? a.blocks - 1 : rank - 1;
     const unsigned down_rank = (int)rank == a.blocks - 1 ? 0 : rank + 1;
@@ -349,8 +395,6 @@ __device__ __forceinline__ void resident_rows(const ResArgs &a, int r0, int w, i
     const bool tell_up = lane == 0 && !top && !up_far, tell_down = lane == 0 && !bottom && !down_far;
     const bool expect = lane == 0 && bytes > 0;
     const bool alone = top && bottom;  // nobody hands this warp a row
-    bool good = true;
-
     float Y[OUT ? NR : 1][V];
     float su[V], sv[V];
     auto react = [&](int q) {
@@ -401,7 +445,7 @@ __device__ __forceinline__ void resident_rows(const ResArgs &a, int r0, int w, i
                 react(q);
             }
         }
-        good = good && (alone || bar_wait(bar + 8 * b, (t >> 1) & 1));  // after a failure no wait, to the end
+        if (!alone && !bar_wait(bar + 8 * b, (t >> 1) & 1, a.wait_ns)) give_up(a, r0, NR, flag);
         float nu[V], nv[V], bu[V], bv[V], nue = 0.0f, nve = 0.0f;  // the handed rows above and below
         const unsigned at = from + b * buf_step;
         hand_load<V>(at, nu);
@@ -437,16 +481,22 @@ __device__ __forceinline__ void resident_rows(const ResArgs &a, int r0, int w, i
         }
     }
 
+    // every warp has done its steps or given up: nothing is handed on from here
+    cluster_arrive();
+    cluster_wait();
+    const bool failed = flag_get(flag);  // the same answer in the whole cluster
+    const float nan = __int_as_float(0x7fffffff);
     if (in_use) {
 #pragma unroll
         for (int q = 0; q < NR; ++q)
 #pragma unroll
             for (int e = 0; e < V; ++e) {
                 const int64_t off = (int64_t)(r0 + q) * a.nm + col + e;
-                a.u[off] = good ? U[q][e] : __int_as_float(0x7fffffff);
-                if constexpr (!OUT) a.v[off] = W[q][e];
+                a.u[off] = failed ? nan : U[q][e];
+                if (!OUT || failed) a.v[off] = failed ? nan : W[q][e];
             }
     }
+    if (failed) drain();
 }
 
 // One cluster; warp g of it holds rows g NN / nwarps .. (g + 1) NN / nwarps - 1.
@@ -469,11 +519,12 @@ k_resident(const ResArgs a) {
         const bool top = BC == BC_MIRROR && g == 0, bottom = BC == BC_MIRROR && g == nwarps - 1;
         const bool up_far = w == 0 && a.blocks > 1, down_far = w == a.warps - 1 && a.blocks > 1;
         const int n = (!top && !up_far) + (!bottom && !down_far) + ((!top && up_far) || (!bottom && down_far));
-        bar_init(bar, max(n, 1));
-        bar_init(bar + 8, max(n, 1));
+        bar_init(bar, max(n, 1) + a.never);
+        bar_init(bar + 8, max(n, 1) + a.never);
+        if (w == 0) asm volatile("st.shared.u32 [%0], %1;" ::"r"(bar + 16 * a.warps), "r"(0u) : "memory");  // no failure
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // every block's mbarriers stand before another hands it a row
+    // every block's mbarriers and flag stand before another hands it a row
     cluster_arrive();
     cluster_wait();
     switch (nr) {  // 1 .. kResRows, chosen by the launcher
@@ -482,9 +533,6 @@ k_resident(const ResArgs a) {
         case 3: resident_rows<V, 3, RX, BC, RAG>(a, r0, w, g, rank, smem); break;
         default: resident_rows<V, 4, RX, BC, RAG>(a, r0, w, g, rank, smem); break;
     }
-    // no block leaves while rows it handed on are on their way
-    cluster_arrive();
-    cluster_wait();
     pdl_trigger();
 }
 

@@ -11,8 +11,8 @@
 namespace rdk {
 
 template <int V>
-constexpr size_t resident_smem(int warps) {  // two parities x two directions x two fields, and the mbarriers
-    return (size_t)2 * warps * 2 * 2 * 128 * V + (size_t)16 * warps;
+constexpr size_t resident_smem(int warps) {  // two parities x two directions x two fields, the mbarriers, the flag
+    return (size_t)2 * warps * 2 * 2 * 128 * V + (size_t)16 * warps + 16;
 }
 
 // The most blocks, 16 or 8, of a cluster of the largest blocks that the current
@@ -61,8 +61,10 @@ bool resident_runs(int blocks, int warps) {
 // `steps` steps of (u, v) in place, or cudaErrorNotSupported with nothing launched.
 template <int V>
 cudaError_t resident_launch_v(int reaction, int boundary, void *u, void *v, int64_t nn, int64_t nm,
-                              const rdcnn_params &p, int blocks, int warps, int64_t steps, cudaStream_t s) {
-    ResArgs a{(float *)u, (float *)v, (int)nn, (int)nm, (int)steps, blocks, warps, make_coef<float>(p, reaction)};
+                              const rdcnn_params &p, int blocks, int warps, int64_t steps, bool give_up,
+                              cudaStream_t s) {
+    ResArgs a{(float *)u, (float *)v, (int)nn, (int)nm, (int)steps, blocks, warps, make_coef<float>(p, reaction),
+              give_up ? kResGiveUpNs : kResWaitNs, give_up ? 1 : 0};
     return with_model(reaction, boundary, [&](auto rx, auto bc) -> cudaError_t {
         constexpr int RX = decltype(rx)::value;
         constexpr int BC = decltype(bc)::value;
@@ -98,4 +100,4 @@ cudaError_t resident_launch_v(int reaction, int boundary, void *u, void *v, int6
 
 #define RDK_RESIDENT_SIG(VV)                                                                                 \
     cudaError_t rdk::resident_launch_v<VV>(int, int, void *, void *, int64_t, int64_t, const rdcnn_params &, \
-                                           int, int, int64_t, cudaStream_t)
+                                           int, int, int64_t, bool, cudaStream_t)

@@ -60,6 +60,41 @@ def test_planes_off_their_alignment_and_captured_runs(rd, shape):
         assert all((t.cpu().numpy() == r).all() for t, r in zip(got, ref))
 
 
+@pytest.mark.parametrize("boundary,reaction", MODELS)
+@pytest.mark.parametrize("shape", [(2, 17), (16, 16), (64, 64), (61, 130), (256, 256), (256, 384), (1024, 100)])
+def test_a_wait_that_gives_up_leaves_no_cell_that_looks_like_a_result(rd, shape, boundary, reaction):
+    """Every wait runs out in the first step (an arrival that nobody makes): the launch ends, both planes
+    are NaN in every cell, and the next run on the same planes gives its bits as ever."""
+    from paper_2102_10340_gb300 import _lib as L
+
+    x, y = (torch.from_numpy(inp.uniform_field(s, *shape)).float().cuda() for s in (44, 45))
+    g = rd.Grid(*shape, _gene(reaction), reaction=reaction, boundary=boundary)
+    g.set_state(x, y)
+    rc = g.lib.rdcnn_run_cluster(g.h, 9, 1)
+    if rc == L.EINVAL and "no room" in L.last_error():
+        pytest.skip("this device runs no cluster of 16 blocks")
+    L.check(rc)
+    torch.cuda.synchronize()
+    assert torch.isnan(g.u).all() and torch.isnan(g.v).all()
+    out = []
+    for run in (lambda: L.check(g.lib.rdcnn_run_cluster(g.h, 9, 0)), lambda: g.run(9, variant="generic")):
+        g.set_state(x, y)
+        run()
+        out.append(g.state())
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+
+
+def test_cluster_runs_are_refused_where_the_grid_does_not_fit(rd):
+    from paper_2102_10340_gb300 import _lib as L
+
+    for shape, dtype in (((64, 15), torch.float32), ((64, 385), torch.float32), ((257, 300), torch.float32),
+                         ((64, 64), torch.float64)):
+        g = rd.Grid(*shape, inp.default_params(), dtype=dtype)
+        assert g.lib.rdcnn_run_cluster(g.h, 1, 0) == L.EINVAL and "fit" in L.last_error()
+    g = rd.Grid(64, 64, inp.default_params())
+    assert g.lib.rdcnn_run_cluster(g.h, -1, 0) == L.EINVAL
+
+
 def test_runs_on_two_streams_at_once(rd):
     """Clusters of two grids on two streams, many short runs each: each grid gets its own bits."""
     out = []

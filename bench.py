@@ -705,6 +705,9 @@ def run_ours(args):
     grid.set_tune(k=tune["k"], rows=tune["rows"])
     variant = tune["variant"]
     plan = grid.plan(variant, tune["k"])  # rows = 0 resolves to the launcher's own choice
+    if variant == "auto":  # time and report the named shape that AUTO stands for at this size
+        tune, variant = dict(tune, **plan), plan["variant"]
+        grid.set_tune(k=tune["k"], rows=tune["rows"])
 
     def barrier():
         if world > 1:

@@ -11,13 +11,17 @@ import torch
 
 _cache: dict = {}
 
-GRID_CANDIDATES_F32 = [("temporal", k, r) for k in (2, 3, 4, 5, 6, 8) for r in (0, 8, 16, 32, 64, 128, 256)] + \
+# the library's own choice, with nothing tuned: FP32 grids of one cluster and FP64 single steps
+# of one and two rows are reached by it (64 x 64, us a step: FP32 0.17 against 0.84 for the best
+# temporal shape, FP64 2.3 against 5.9)
+AUTO = ("auto", 0, 0)
+GRID_CANDIDATES_F32 = [AUTO] + [("temporal", k, r) for k in (2, 3, 4, 5, 6, 8) for r in (0, 8, 16, 32, 64, 128, 256)] + \
                       [("temporal2", k, r) for k in (4, 6, 8) for r in (0, 64, 176, 256)] + \
                       [("temporal_wide", k, r) for k in (2, 3, 4) for r in (0, 32, 64, 128)] + \
-                      [("step1", 1, r) for r in (4, 8, 16, 32)]
-GRID_CANDIDATES_F64 = [("temporal", k, r) for k in (2, 3, 4) for r in (0, 32, 64, 128)] + \
+                      [("step1", 1, r) for r in (1, 2, 4, 8, 16, 32)]
+GRID_CANDIDATES_F64 = [AUTO] + [("temporal", k, r) for k in (2, 3, 4) for r in (0, 32, 64, 128)] + \
                       [("temporal2", k, r) for k in (2, 4) for r in (0, 64)] + \
-                      [("step1", 1, r) for r in (4, 8, 16)]
+                      [("step1", 1, r) for r in (1, 2, 4, 8, 16)]
 # 256-row strips won at the 256-instance sweep with four-warp blocks (k = 4: 1156 against 1130
 # Gcell/s at 128 rows), 128-row strips with one-warp blocks (1298); 96 and 192 lie between
 BATCH_CANDIDATES = [(k, r) for k in (2, 3, 4, 6, 8) for r in (16, 32, 64, 96, 128, 192, 256, 512)]
@@ -37,7 +41,8 @@ def _time(fn, reps: int = 2) -> float:
 
 
 def tune_grid(grid, x=None, trial_steps: int = 48, force: bool = False) -> dict:
-    """Best {variant, k, rows} for this grid's size and dtype (cached)."""
+    """Best {variant, k, rows} for this grid's size and dtype (cached); {"auto", 0, 0} is the
+    library's own choice, with nothing tuned.  The grid timed here is left with that k and rows."""
     key = ("grid", grid.nn, grid.nm, grid.dtype, grid.reaction, getattr(grid, "boundary", "periodic"))
     if key in _cache and not force:
         return dict(_cache[key])

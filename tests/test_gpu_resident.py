@@ -84,6 +84,17 @@ def test_a_wait_that_gives_up_leaves_no_cell_that_looks_like_a_result(rd, shape,
     assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
 
 
+def test_a_tuned_grid_still_runs_in_one_launch(rd):
+    """The tuner finds the cluster launch of a small FP32 grid and leaves it in force."""
+    from paper_2102_10340_gb300 import autotune
+
+    g = rd.Grid(64, 64, inp.default_params())
+    best = autotune.tune_grid(g, torch.from_numpy(inp.uniform_field(46, 64, 64)).float().cuda(), force=True)
+    before = rd.launch_count()
+    g.run(500, variant=best["variant"], k=best["k"])
+    assert best["variant"] == "auto" and rd.launch_count() - before == 1
+
+
 def test_cluster_runs_are_refused_where_the_grid_does_not_fit(rd):
     from paper_2102_10340_gb300 import _lib as L
 

@@ -195,8 +195,8 @@ int rdcnn_set_state(rdcnn_t *h, const void *u0, const void *v0, int on_device);
  * variants need NM to be a multiple of 4 (F32, BF16, F16) or 2 (F64) and
  * 16-byte (8-byte for BF16 / F16) aligned buffers;
  * otherwise an explicit request returns RDCNN_EINVAL, and AUTO runs F32
- * planes through the temporal pipeline with elements copied one by one, others
- * through GENERIC.  AUTO on F64 planes is STEP1 unless a depth is asked for
+ * planes through the temporal pipeline with elements copied one by one (unless
+ * they are too narrow for it), others through GENERIC.  AUTO on F64 planes is STEP1 unless a depth is asked for
  * (k or tune->k).  AUTO on F32 grids of 16 to 384 columns and up to 1024 (129
  * columns and more: 512, 257 and more: 256) rows, with no k and no tune,
  * advances whole stretches of the run in one launch of one thread-block

@@ -341,7 +341,8 @@ int run_core(rdcnn_t *h, int64_t T, int variant, int k, int64_t every, MarkFn ma
     // launch; FP64 planes are fastest with one (auto_single_step).  A depth that
     // only the vectorised variants would reject is ignored here, as GENERIC
     // ignores it.
-    if (autov && variant == RDCNN_VARIANT_GENERIC && h->dtype == RDCNN_F32) {
+    if (autov && variant == RDCNN_VARIANT_GENERIC && h->dtype == RDCNN_F32 &&
+        ragged_pays(h->nn, h->nm, every > 0 ? std::min(every, T) : T)) {
         variant = kVariantRagged;
         k = (k_arg >= 1 && k_arg <= max_k(h->dtype)) ? k_arg : h->tune_k ? h->tune_k : default_k_ragged(h->nn, h->nm);
     }

@@ -288,6 +288,20 @@ int auto_rows_f32(bool ragged, int K, int64_t nn, int64_t nm) {
     return model_rows(ragged ? kRaggedBeats : kBeats, K, nn, nm, &us);
 }
 
+// Whether AUTO steps FP32 rows that are no lane vectors through the pipeline
+// rather than one thread a cell.  The pipeline's warps are 128 columns wide
+// whatever the grid's width, so narrow tall grids are better off with threads,
+// the more so the fewer steps there are (a pass over memory then advances few of
+// them, and one or two also need fuller bands).  us for 24 steps, threads /
+// pipeline: 200000 x 1 62 / 1080, 200000 x 3 127 / 511, 100000 x 13 225 / 223, 100000 x
+// 17 269 / 224, 1025 x 3 54 / 33; 3 steps: 400000 x 21 161 / 197; 2 steps: 100000 x 17 22 / 48,
+// 100000 x 45 51 / 50, 20000 x 121 29 / 42, 20000 x 225 51 / 43; 1 step: 100000 x 65 50 / 57.
+bool ragged_pays(int64_t nn, int64_t nm, int64_t steps) {
+    if (steps > 2) return (nm - 13) * steps >= 38 || nn <= 900 * nm;
+    const int64_t bands = (nm + 119) / 120;
+    return nm >= (bands > 1 ? 95 * bands : steps == 2 ? 50 : 75);
+}
+
 // Rows per warp strip when the caller gives none (FP64 and 16-bit planes, 8
 // values per lane, warp pairs).  Small grids use short strips (few warps exist at all); large grids pick, among a few lengths,
 // the one that minimises waves x (rows + 2K) -- the work of the slowest SM

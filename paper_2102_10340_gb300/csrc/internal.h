@@ -145,6 +145,8 @@ cudaError_t launch_temporal_wide(int dtype, int reaction, int boundary, int k, c
 cudaError_t launch_temporal_ragged(int reaction, int boundary, int k, const void *u,
                                    const void *v, void *un, void *vn, int64_t nn, int64_t nm,
                                    const rdcnn_params &p, int rows, cudaStream_t s);
+// Whether AUTO takes it for a run, or the stretch to a mark, of that many steps.
+bool ragged_pays(int64_t nn, int64_t nm, int64_t steps);
 // The temporal pipeline with the K stages split across a warp pair (k >= 2;
 // FP32 / FP64 planes, every model).
 cudaError_t launch_temporal_split(int dtype, int reaction, int boundary, int k, const void *u, const void *v,

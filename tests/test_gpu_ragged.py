@@ -43,3 +43,23 @@ def test_every_depth_on_misaligned_planes(rd, dtype, k):
         assert all(float(t[0]) == 0.0 and float(t[-1]) == 0.0 for t in base)
         out.append((u.clone(), v.clone()))
     assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("shape,T,single", [((900, 1), 3, False), ((901, 1), 3, True), ((12600, 14), 24, False),
+                                            ((12601, 14), 24, True), ((20000, 15), 24, False), ((23000, 25), 3, True),
+                                            ((24000, 26), 3, False), ((2000, 49), 2, None), ((2000, 50), 2, None),
+                                            ((2000, 74), 1, None), ((2000, 75), 1, None), ((1100, 189), 2, None),
+                                            ((1100, 191), 2, None)])
+def test_narrow_grids_take_one_thread_a_cell(rd, shape, T, single):
+    """On both sides of the rule: as many launches as steps, or fewer (one or two steps take as many
+    launches either way), and the same bits."""
+    x, y = (torch.from_numpy(inp.uniform_field(s, *shape)).float().cuda() for s in (34, 35))
+    out = []
+    for variant in ("auto", "generic"):
+        g = rd.Grid(*shape, inp.default_params())
+        g.set_state(x, y)
+        before = rd.launch_count()
+        g.run(T, variant=variant)
+        out.append((rd.launch_count() - before, *g.state()))
+    assert torch.equal(out[0][1], out[1][1]) and torch.equal(out[0][2], out[1][2])
+    assert out[1][0] == T and (single is None or (out[0][0] == T) == single)

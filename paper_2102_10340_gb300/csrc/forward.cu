@@ -256,9 +256,10 @@ int model_rows(const BeatModel &m, int K, int64_t nn, int64_t nm, double *us) {
     const int64_t bands = (nm + (32 - 2 * H) * 4 - 1) / ((32 - 2 * H) * 4);
     const int64_t slots = (int64_t)sm_count() * 8;
     int best = 1;
+    int64_t strips = 0;
     *us = 1e300;
-    for (int w = 0; w <= 8; ++w) {  // w = 0: one warp per scheduler
-        const int64_t strips = std::min<int64_t>((w ? w * slots : slots / 2) / bands, (nn + 1) / 2);
+    for (int w = 0; w <= 8 && strips < (nn + 1) / 2; ++w) {  // w = 0: one warp per scheduler
+        strips = std::min<int64_t>((w ? w * slots : slots / 2) / bands, (nn + 1) / 2);
         if (strips < 1) continue;
         const int64_t rows = (nn + strips - 1) / strips;
         const double t = launch_us(m, K, bands * ((nn + rows - 1) / rows), rows, slots);
@@ -286,6 +287,22 @@ double temporal_us(int K, int64_t warps, int64_t rows, int sms) { return launch_
 int auto_rows_f32(bool ragged, int K, int64_t nn, int64_t nm) {
     double us;
     return model_rows(ragged ? kRaggedBeats : kBeats, K, nn, nm, &us);
+}
+
+// Depths up to 4 of grids whose four planes do not fit L2 together are bound by
+// DRAM, not by the beats of the model: fastest with short strips at depths 1 and
+// 2, and with one wave of 12 warps an SM at 3 and 4 (at 4, 16 where registers allow
+// that many).  us a step, strips before the model / by the model / now: 8192^2 depth 1
+// 194 / 184 / 169, 3 59 / 65 / 59, 4 48 / 60 / 44, zero flux 48 / 45 / 45; 6000^2 1 101 /
+// 107 / 93, 4 24.9 / 26.1 / 24.8, zero flux 24.9 / 28.9 / 24.7; 4096^2 1 49 / 52 / 46, 4
+// 13.2 / 12.9 / 11.8; 2900 x 3128 1 25.6 / 29.0 / 24.7.
+bool beyond_l2(int64_t nn, int64_t nm) { return nn * nm >= 6000000; }
+int dram_rows_f32(int K, int64_t nn, int64_t nm, int warps_per_sm) {
+    if (K == 1) return 10;
+    if (K == 2) return 12;
+    if (K == 3 && nn * nm >= (int64_t(1) << 27)) return 20;
+    const int64_t strips = (int64_t)warps_per_sm * sm_count() / ((nm + 119) / 120);
+    return (int)(strips < 1 ? std::min<int64_t>(nn, 128) : (nn + strips - 1) / strips);
 }
 
 // Whether AUTO steps FP32 rows that are no lane vectors through the pipeline

@@ -184,6 +184,9 @@ int auto_rows_temporal(int K, int64_t nn, int64_t nm, int bands, int blocks_per_
                        int warps_per_block);
 // The same for FP32 planes with 4 values per lane (launch model in forward.cu).
 int auto_rows_f32(bool ragged, int K, int64_t nn, int64_t nm);
+// Depths 1 .. 4 of grids beyond L2, with that many resident warps an SM.
+bool beyond_l2(int64_t nn, int64_t nm);
+int dram_rows_f32(int K, int64_t nn, int64_t nm, int warps_per_sm);
 // us of an FP32 temporal launch of depth K with that many strips of that many
 // rows on a device of `sms` SMs.
 double temporal_us(int K, int64_t warps, int64_t rows, int sms);

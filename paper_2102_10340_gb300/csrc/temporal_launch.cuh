@@ -3,6 +3,8 @@
 // (dtype, K, reaction, boundary) kernels compile in parallel.
 #pragma once
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "internal.h"
 #include "temporal.cuh"
@@ -33,8 +35,20 @@ constexpr int temporal_bands(int64_t nm) {
 template <typename T, int K>
 int temporal_rows(int reaction, int boundary, int64_t nn, int64_t nm, int rows) {
     if (rows > 0) return rows;
-    if constexpr (std::is_same<T, float>::value || IsRagged<T>::value) return auto_rows_f32(IsRagged<T>::value, K, nn, nm);
     int r = 0;
+    if constexpr (std::is_same<T, float>::value && K <= 4) {
+        if (beyond_l2(nn, nm)) {
+            int warps = 12;
+            if constexpr (K == 4)
+                with_model(reaction, boundary, [&](auto rx, auto bc) {
+                    warps = std::max(4, temporal_blocks_per_sm<T, K, decltype(rx)::value, decltype(bc)::value>() *
+                                            kTemporalWarps / 4 * 4);
+                    return cudaSuccess;
+                });
+            return dram_rows_f32(K, nn, nm, warps);
+        }
+    }
+    if constexpr (std::is_same<T, float>::value || IsRagged<T>::value) return auto_rows_f32(IsRagged<T>::value, K, nn, nm);
     with_model(reaction, boundary, [&](auto rx, auto bc) {
         r = auto_rows_temporal(K, nn, nm, temporal_bands<T, K>(nm),
                                temporal_blocks_per_sm<T, K, decltype(rx)::value, decltype(bc)::value>(),

@@ -146,3 +146,27 @@ def test_captured_states_and_odd_runs(rd):
     graph.replay()
     torch.cuda.synchronize()
     assert torch.equal(g.u, h.u) and torch.equal(g.v, h.v)
+
+
+@pytest.mark.parametrize("boundary,reaction", [("periodic", "fhn"), ("zeroflux", "fhn"), ("periodic", "cenn")])
+def test_strips_beyond_l2(rd, boundary, reaction):
+    """Strips of depths 1 to 4 from six million cells on: their lengths, whole waves at depths 3 and 4, and
+    the bits of the one-thread-per-cell kernel."""
+    gene = {"dt": 0.1, "a": 0.0, "b": 0.0, "eps": 0.0, "c": 1.3, "Du": 0.2, "Dv": 0.0} if reaction == "cenn" \
+        else inp.default_params()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    nn, nm = 2600, 2400  # 20 bands
+    x = torch.rand((nn, nm), generator=torch.Generator(device="cuda").manual_seed(5), device="cuda") * 2 - 1
+    ref = rd.Grid(nn, nm, gene, boundary=boundary, reaction=reaction)
+    ref.set_state(x, -x).run(12, variant="generic")
+    for k in (1, 2, 3, 4):
+        g = rd.Grid(nn, nm, gene, boundary=boundary, reaction=reaction)
+        rows = g.plan("temporal", k)["rows"]
+        if k < 3:
+            assert rows == (10, 12)[k - 1]
+        else:
+            assert any(rows == -(-nn // (p * sms // 20)) for p in ((12,) if k == 3 else (4, 8, 12, 16, 20)))
+        g.set_state(x, -x).run(12, variant="temporal", k=k)
+        assert torch.equal(g.u, ref.u) and torch.equal(g.v, ref.v), k
+    small = rd.Grid(2400, 2400, gene, boundary=boundary, reaction=reaction)  # 5.76 million: the launch model
+    assert small.plan("temporal", 1)["rows"] != 10

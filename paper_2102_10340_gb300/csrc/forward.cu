@@ -32,6 +32,7 @@
 // (k_temporal_split) in split_launch.cuh and the split_*.cu units; they
 // compile in parallel.
 #include <algorithm>
+#include <atomic>
 
 #include "common.cuh"
 #include "internal.h"
@@ -365,10 +366,16 @@ cudaError_t generic_t(int reaction, int boundary, const void *u, const void *v, 
 }  // namespace
 
 int sm_count() {
+    static std::atomic<int> known[64];  // by device
     int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0)
-        return n;
+    if (cudaGetDevice(&dev) == cudaSuccess) {
+        if (dev < 64 && (n = known[dev].load(std::memory_order_relaxed)) > 0) return n;
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0) {
+            if (dev < 64) known[dev].store(n, std::memory_order_relaxed);
+            return n;
+        }
+    }
+    (void)cudaGetLastError();
     return 152;
 }
 

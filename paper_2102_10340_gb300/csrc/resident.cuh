@@ -34,8 +34,8 @@
 // Waits are bounded.  A warp whose wait gives up sets a flag in every block and
 // ends (give_up): it hands on no more rows, so its neighbours' waits give up in
 // turn.  The flag is read after the barrier that ends the steps, and every warp
-// of the cluster then stores NaNs in both planes: a failed run has no cell that
-// looks like a result.
+// of the cluster then stores NaNs in both planes, over its rows: a failed run has
+// no cell that looks like a result.
 //
 // Bound: latency of the hand-over up to 128^2 (64^2: 370 cycles a step, of which
 // about 100 are the sums and the update), one warp's issue rate per scheduler of
@@ -205,8 +205,13 @@ __device__ __forceinline__ bool flag_get(unsigned flag) {
     asm volatile("ld.shared.u32 %0, [%1];" : "=r"(x) : "r"(flag) : "memory");
     return x != 0;
 }
-// Rows that nobody waited for may still be on their way: no block leaves before they are in.
-__device__ __forceinline__ void drain() {
+// After a failure: NaNs in the warp's rows, over what it has stored.  Handed rows that
+// nobody waited for may still be on their way: no block leaves before they are in.
+__device__ __forceinline__ void spoil(const ResArgs &a, int r0, int nr) {
+    __syncwarp();
+#pragma unroll 1
+    for (int i = threadIdx.x & 31; i < nr * a.nm; i += 32)
+        a.u[(int64_t)r0 * a.nm + i] = a.v[(int64_t)r0 * a.nm + i] = __int_as_float(0x7fffffff);
     const uint64_t t0 = clock_ns();
     while (!__any_sync(kFull, clock_ns() - t0 >= kResDrainNs)) {}
     cluster_arrive();
@@ -225,11 +230,7 @@ __device__ __forceinline__ void give_up(const ResArgs &a, int r0, int nr, unsign
     __syncwarp();
     cluster_arrive();
     cluster_wait();
-#pragma unroll 1
-    for (int i = lane; i < nr * a.nm; i += 32)
-        a.u[(int64_t)r0 * a.nm + i] = a.v[(int64_t)r0 * a.nm + i] = __int_as_float(0x7fffffff);
-    __syncwarp();
-    drain();
+    spoil(a, r0, nr);
     asm volatile("{\n.reg .pred q;\nsetp.ne.u32 q, %0, 0;\n@q exit;\n}" ::"r"(a.blocks) : "memory");
 }
 template <int V>
@@ -481,22 +482,20 @@ __device__ __forceinline__ void resident_rows(const ResArgs &a, int r0, int w, i
         }
     }
 
-    // every warp has done its steps or given up: nothing is handed on from here
-    cluster_arrive();
-    cluster_wait();
-    const bool failed = flag_get(flag);  // the same answer in the whole cluster
-    const float nan = __int_as_float(0x7fffffff);
     if (in_use) {
 #pragma unroll
         for (int q = 0; q < NR; ++q)
 #pragma unroll
             for (int e = 0; e < V; ++e) {
                 const int64_t off = (int64_t)(r0 + q) * a.nm + col + e;
-                a.u[off] = failed ? nan : U[q][e];
-                if (!OUT || failed) a.v[off] = failed ? nan : W[q][e];
+                a.u[off] = U[q][e];
+                if constexpr (!OUT) a.v[off] = W[q][e];
             }
     }
-    if (failed) drain();
+    // every warp has done its steps or given up: nothing is handed on from here
+    cluster_arrive();
+    cluster_wait();
+    if (flag_get(flag)) spoil(a, r0, NR);  // the same answer in the whole cluster
 }
 
 // One cluster; warp g of it holds rows g NN / nwarps .. (g + 1) NN / nwarps - 1.

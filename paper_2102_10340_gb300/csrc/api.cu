@@ -368,7 +368,9 @@ int run_core(rdcnn_t *h, int64_t T, int variant, int k, int64_t every, MarkFn ma
         if (left == 0) return RDCNN_OK;
     }
     // FP32 bits do not depend on the depth of a launch: without one asked for, it is free
-    const bool own_depth = autov && k_arg == 0 && h->tune_k == 0 && h->dtype == RDCNN_F32;
+    const bool own_depth = autov && k_arg == 0 && h->tune_k == 0 && h->dtype == RDCNN_F32 &&
+                           variant != RDCNN_VARIANT_GENERIC;
+    int64_t launches = 0;  // to come in the present stretch
     // launch-bound runs: replay whole groups of full-depth launches as a graph
     const int64_t full = left / k;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -392,9 +394,11 @@ int run_core(rdcnn_t *h, int64_t T, int variant, int k, int64_t every, MarkFn ma
             // the launches up to the end or the next mark, of even depth rather than
             // full ones and a rest; up to the end, as many as end in (u, v)
             const int64_t stretch = every > 0 ? std::min<int64_t>(left, every - done % every) : left;
-            int64_t n = (stretch + k - 1) / k;
-            if (every == 0 && (n % 2 == 0) != (cu == h->u) && n < stretch) ++n;
-            kk = (int)((stretch + n - 1) / n);
+            if (launches == 0)
+                launches = stretch_launches(variant == kVariantRagged, h->nn, h->nm, stretch, k,
+                                            every > 0 ? -1 : cu == h->u ? 0 : 1);
+            kk = (int)((stretch + launches - 1) / launches);
+            --launches;
         }
         const bool marks = every > 0 && (done + kk) % every == 0;
         void *du = nullptr, *dv = nullptr;

@@ -306,6 +306,50 @@ int dram_rows_f32(int K, int64_t nn, int64_t nm, int warps_per_sm) {
     return (int)(strips < 1 ? std::min<int64_t>(nn, 128) : (nn + strips - 1) / strips);
 }
 
+// us of an FP32 temporal launch at the strips it gets, and of a copy of the state.
+namespace {
+double launch_cost(bool ragged, int K, int64_t nn, int64_t nm) {
+    const double pass = (double)(nn * nm) * 16;  // bytes of one over the planes
+    if (beyond_l2(nn, nm) && K <= 4) return pass / (K == 1 ? 6.4e6 : 6.0e6);
+    double us;
+    (void)model_rows(ragged ? kRaggedBeats : kBeats, K, nn, nm, &us);
+    if (!beyond_l2(nn, nm)) return us;
+    const double dram = pass / 6.2e6;
+    return std::max(us, dram) + 0.25 * std::min(us, dram);
+}
+// Planes that are no whole vectors are copied one after the other.
+double copy_cost(int64_t nn, int64_t nm) {
+    return (nn * nm % 4 != 0 ? 10.0 : 1.7) + (double)(nn * nm) * 16 / (beyond_l2(nn, nm) ? 6.7e6 : 12e6);
+}
+constexpr double kHostUs = 2.9;  // the host's share of a launch
+}  // namespace
+
+// A stretch of up to 16 steps takes as many launches as cost least, the copy of a
+// state that ends in the scratch planes included; a longer one launches of the
+// default depth k.  home: what the parity of the number of launches must be for
+// the state to end where it belongs (0 even, 1 odd; -1: anywhere).  us, launches of
+// at most depth k, even in number / as here: 512^2 9 steps 18.5 / 13.4, 1024^2 9 steps 20.0 /
+// 17.6, 8192^2 3 steps 375 / 341, 200000 x 4 2 steps 91 / 60.
+int64_t stretch_launches(bool ragged, int64_t nn, int64_t nm, int64_t steps, int k, int home, double *us) {
+    const BeatModel &m = ragged ? kRaggedBeats : kBeats;
+    int64_t n = (steps + k - 1) / k;
+    auto strays = [&](int64_t c) { return home >= 0 && c % 2 != home; };
+    if (steps > 2 * m.k1) {
+        if (strays(n) && n < steps) ++n;
+        if (us) *us = (double)n * std::max(kHostUs, launch_cost(ragged, (int)((steps + n - 1) / n), nn, nm));
+        return n;
+    }
+    double least = 1e300;
+    int64_t best = n;
+    for (int64_t c = (steps + m.k1 - 1) / m.k1; c <= std::min(steps, n + (strays(n) ? 1 : 0)); ++c) {
+        const double t = (double)c * std::max(kHostUs, launch_cost(ragged, (int)((steps + c - 1) / c), nn, nm)) +
+                         (strays(c) ? std::max(kHostUs, copy_cost(nn, nm)) : 0.0);
+        if (t <= least) { least = t; best = c; }
+    }
+    if (us) *us = least;
+    return best;
+}
+
 // Whether AUTO steps FP32 rows that are no lane vectors through the pipeline
 // rather than one thread a cell.  The pipeline's warps are 128 columns wide
 // whatever the grid's width, so narrow tall grids are better off with threads,

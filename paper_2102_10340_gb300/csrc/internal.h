@@ -190,6 +190,9 @@ int dram_rows_f32(int K, int64_t nn, int64_t nm, int warps_per_sm);
 // us of an FP32 temporal launch of depth K with that many strips of that many
 // rows on a device of `sms` SMs.
 double temporal_us(int K, int64_t warps, int64_t rows, int sms);
+// Launches that AUTO divides a stretch of `steps` FP32 steps into (default depth
+// k), and what they take.
+int64_t stretch_launches(bool ragged, int64_t nn, int64_t nm, int64_t steps, int k, int home, double *us = nullptr);
 // u = v = ka * x; x may alias u.
 cudaError_t launch_init(int dtype, const void *x, void *u, void *v, double ka, int64_t n,
                         cudaStream_t s);

@@ -170,3 +170,17 @@ def test_strips_beyond_l2(rd, boundary, reaction):
         assert torch.equal(g.u, ref.u) and torch.equal(g.v, ref.v), k
     small = rd.Grid(2400, 2400, gene, boundary=boundary, reaction=reaction)  # 5.76 million: the launch model
     assert small.plan("temporal", 1)["rows"] != 10
+
+
+@pytest.mark.parametrize("shape,T,launches", [((512, 512), 9, 2), ((1024, 1024), 10, 2), ((2600, 2400), 3, 1),
+                                              ((2600, 2400), 8, 2), ((509, 515), 9, 2)])
+def test_launches_of_short_stretches(rd, shape, T, launches):
+    """Few deep launches, or one and a copy of the state, where more launches would cost more; the same bits."""
+    x = torch.rand(shape, generator=torch.Generator(device="cuda").manual_seed(6), device="cuda") * 2 - 1
+    g, h = (rd.Grid(*shape, inp.default_params()) for _ in range(2))
+    g.set_state(x, -x)
+    before = rd.launch_count()
+    g.run(T)
+    assert rd.launch_count() - before == launches
+    h.set_state(x, -x).run(T, variant="generic")
+    assert torch.equal(g.u, h.u) and torch.equal(g.v, h.v)

@@ -352,7 +352,9 @@ int run_core(rdcnn_t *h, int64_t T, int variant, int k, int64_t every, MarkFn ma
     // small FP32 grids with no depth or strip length asked for: whole stretches of
     // the run in one launch, in place
     if (autov && k_arg == 0 && h->tune_k == 0 && h->tune_rows == 0 && h->dtype == RDCNN_F32 &&
-        resident_fits(h->nn, h->nm)) {
+        resident_fits(h->nn, h->nm) &&
+        resident_pays(h->boundary, h->nn, h->nm, every > 0 ? std::min(every, T) : T, every > 0,
+                      variant != RDCNN_VARIANT_TEMPORAL, k)) {
         while (left > 0) {
             int64_t n = std::min<int64_t>(left, kResidentSteps);
             if (every > 0) n = std::min<int64_t>(n, every - (T - left) % every);

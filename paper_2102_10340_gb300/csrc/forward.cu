@@ -321,7 +321,6 @@ double launch_cost(bool ragged, int K, int64_t nn, int64_t nm) {
 double copy_cost(int64_t nn, int64_t nm) {
     return (nn * nm % 4 != 0 ? 10.0 : 1.7) + (double)(nn * nm) * 16 / (beyond_l2(nn, nm) ? 6.7e6 : 12e6);
 }
-constexpr double kHostUs = 2.9;  // the host's share of a launch
 }  // namespace
 
 // A stretch of up to 16 steps takes as many launches as cost least, the copy of a

@@ -160,6 +160,10 @@ cudaError_t launch_temporal_split(int dtype, int reaction, int boundary, int k, 
 // millisecond.
 constexpr int64_t kResidentSteps = 8192;  // most steps of one launch: 1 .. 7 ms
 bool resident_fits(int64_t nn, int64_t nm);
+// Whether such launches beat the temporal ones of default depth k (ragged: on
+// rows that are no lane vectors) for a run, or stretches up to a mark, of
+// `steps` steps.
+bool resident_pays(int boundary, int64_t nn, int64_t nm, int64_t steps, bool marks, bool ragged, int k);
 cudaError_t launch_resident(int reaction, int boundary, void *u, void *v, int64_t nn, int64_t nm,
                             const rdcnn_params &p, int64_t steps, cudaStream_t s, bool give_up = false);
 cudaError_t launch_generic(int dtype, int reaction, int boundary, const void *u, const void *v,
@@ -192,6 +196,7 @@ int dram_rows_f32(int K, int64_t nn, int64_t nm, int warps_per_sm);
 double temporal_us(int K, int64_t warps, int64_t rows, int sms);
 // Launches that AUTO divides a stretch of `steps` FP32 steps into (default depth
 // k), and what they take.
+constexpr double kHostUs = 2.9;  // the host's share of a launch
 int64_t stretch_launches(bool ragged, int64_t nn, int64_t nm, int64_t steps, int k, int home, double *us = nullptr);
 // u = v = ka * x; x may alias u.
 cudaError_t launch_init(int dtype, const void *x, void *u, void *v, double ka, int64_t n,

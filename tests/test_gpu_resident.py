@@ -1,7 +1,7 @@
-"""AUTO on FP32 grids up to 384 columns wide (one cluster holds the state, one launch a stretch of
-steps) against the one-thread-per-cell kernel: the same bits, at the edges of every lane width (2, 4,
+"""FP32 grids up to 384 columns wide held by one cluster (rdcnn_run_cluster, and AUTO where it is the
+faster way) against the one-thread-per-cell kernel: the same bits, at the edges of every lane width (2, 4,
 8 and 12 columns a lane, with a last lane that overlaps the one before it), with 1 to 4 rows a warp, one
-to sixteen blocks, and on both sides of the range's ends."""
+to sixteen blocks; and which launches AUTO takes, on both sides of the range's ends."""
 import pytest
 import torch
 
@@ -14,6 +14,7 @@ SHAPES = [(1, 16), (1, 64), (2, 17), (5, 96), (15, 15), (16, 16), (17, 63), (31,
           (64, 64), (100, 128), (129, 127), (200, 250), (255, 251), (256, 256), (260, 255), (512, 256), (513, 256),
           (1023, 49), (1024, 100), (1025, 64), (1, 257), (17, 268), (48, 257),
           (90, 383), (64, 384), (256, 260), (256, 384), (257, 300), (40, 385)]
+OUTSIDE = [(15, 15), (513, 256), (1025, 64), (257, 300), (40, 385)]  # SHAPES that no cluster holds
 MODELS = [("periodic", "fhn"), ("zeroflux", "fhn"), ("periodic", "cenn"), ("zeroflux", "cenn"), ("zeroflux", "none")]
 
 
@@ -22,14 +23,72 @@ def _gene(reaction):
         else inp.default_params()
 
 
+def _cluster(g, T, give_up=0):
+    """T steps by cluster launches; skips on a device that has no room for sixteen blocks."""
+    from paper_2102_10340_gb300 import _lib as L
+
+    rc = g.lib.rdcnn_run_cluster(g.h, T, give_up)
+    if rc == L.EINVAL and "no room" in L.last_error():
+        pytest.skip("this device runs no cluster of 16 blocks")
+    L.check(rc)
+
+
 @pytest.mark.parametrize("shape", SHAPES)
 @pytest.mark.parametrize("boundary,reaction", MODELS)
-def test_auto_matches_generic_bitwise(rd, shape, boundary, reaction):
-    x, y = inp.uniform_field(41, *shape), 0.7 * inp.uniform_field(42, *shape)
-    for T in (1, 2, 3, 30):
-        a, b = (gpu_run(rd, x, y, _gene(reaction), T, torch.float32, v, reaction=reaction, boundary=boundary)
-                for v in ("auto", "generic"))
-        assert (a[0] == b[0]).all() and (a[1] == b[1]).all(), T
+def test_cluster_and_auto_match_generic_bitwise(rd, shape, boundary, reaction):
+    x, y = (torch.from_numpy(s * inp.uniform_field(i, *shape)).float().cuda() for i, s in ((41, 1.0), (42, 0.7)))
+    for T in (1, 2, 3, 30, 150):
+        out = []
+        for how in ("generic", "auto", "cluster"):
+            g = rd.Grid(*shape, _gene(reaction), reaction=reaction, boundary=boundary)
+            g.set_state(x, y)
+            before = rd.launch_count()
+            if how != "cluster":
+                g.run(T, variant=how)
+            elif shape not in OUTSIDE:
+                _cluster(g, T)
+                assert rd.launch_count() - before == 1
+            else:
+                continue
+            out.append(g.state())
+        assert all(torch.equal(a, b) for o in out[1:] for a, b in zip(o, out[0])), T
+
+
+@pytest.mark.parametrize("shape,T,launches", [((1, 16), 30, 1), ((64, 64), 1, 1), ((64, 64), 30, 1), ((64, 15), 30, None),
+                                              ((1024, 64), 30, 1), ((1025, 64), 30, None), ((512, 256), 8, 2),
+                                              ((512, 256), 300, 1), ((513, 256), 300, None), ((256, 384), 100, 1),
+                                              ((257, 384), 100, None), ((256, 385), 100, None), ((400, 256), 6, 2),
+                                              ((251, 253), 30, 1), ((64, 64), 8192 + 3, 2)])
+def test_which_launches_auto_takes(rd, shape, T, launches):
+    """One launch (of at most 8192 steps) for a whole run in the cluster's range, more than one outside it
+    and for short runs of its largest grids; the same state as in calls of 101 steps."""
+    x = torch.from_numpy(inp.uniform_field(47, *shape)).float().cuda()
+    g, h = (rd.Grid(*shape, inp.default_params()) for _ in range(2))
+    _cluster(rd.Grid(16, 16, inp.default_params()), 1)
+    g.set_state(x, -x)
+    h.set_state(x, -x)
+    before = rd.launch_count()
+    g.run(T)
+    made = rd.launch_count() - before
+    assert made == launches if launches else made > 1
+    for t in range(0, T, 101):
+        h.run(min(101, T - t), variant="generic")
+    assert torch.equal(g.u, h.u) and torch.equal(g.v, h.v)
+
+
+@pytest.mark.parametrize("shape,every,launches", [((256, 256), 1, 10), ((512, 256), 4, 10), ((64, 64), 30, 10)])
+def test_snapshots_between_cluster_and_launches(rd, shape, every, launches):
+    """Every few steps kept: a launch each, written where they are kept; many: a cluster launch each."""
+    x = torch.from_numpy(inp.uniform_field(48, *shape)).float().cuda()
+    g, h = (rd.Grid(*shape, inp.default_params()) for _ in range(2))
+    g.set_state(x, -x)
+    h.set_state(x, -x)
+    before = rd.launch_count()
+    us, vs = g.run_snapshots(10 * every, every, out="device")
+    assert rd.launch_count() - before == launches
+    for s in range(11):
+        assert torch.equal(us[s], h.u) and torch.equal(vs[s], h.v), s
+        h.run(every, variant="generic")
 
 
 @pytest.mark.parametrize("shape", [(64, 64), (37, 121), (256, 256)])
@@ -65,19 +124,14 @@ def test_planes_off_their_alignment_and_captured_runs(rd, shape):
 def test_a_wait_that_gives_up_leaves_no_cell_that_looks_like_a_result(rd, shape, boundary, reaction):
     """Every wait runs out in the first step (an arrival that nobody makes): the launch ends, both planes
     are NaN in every cell, and the next run on the same planes gives its bits as ever."""
-    from paper_2102_10340_gb300 import _lib as L
-
     x, y = (torch.from_numpy(inp.uniform_field(s, *shape)).float().cuda() for s in (44, 45))
     g = rd.Grid(*shape, _gene(reaction), reaction=reaction, boundary=boundary)
     g.set_state(x, y)
-    rc = g.lib.rdcnn_run_cluster(g.h, 9, 1)
-    if rc == L.EINVAL and "no room" in L.last_error():
-        pytest.skip("this device runs no cluster of 16 blocks")
-    L.check(rc)
+    _cluster(g, 9, give_up=1)
     torch.cuda.synchronize()
     assert torch.isnan(g.u).all() and torch.isnan(g.v).all()
     out = []
-    for run in (lambda: L.check(g.lib.rdcnn_run_cluster(g.h, 9, 0)), lambda: g.run(9, variant="generic")):
+    for run in (lambda: _cluster(g, 9), lambda: g.run(9, variant="generic")):
         g.set_state(x, y)
         run()
         out.append(g.state())

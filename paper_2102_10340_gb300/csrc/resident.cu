@@ -72,7 +72,7 @@ bool resident_pays(int boundary, int64_t nn, int64_t nm, int64_t steps, bool mar
     double us;
     const int64_t n = stretch_launches(ragged, nn, nm, steps, k, marks ? -1 : 0, &us);
     if (marks) return std::max(2 * kHostUs, cluster + 1.8) <= std::max((double)n * kHostUs, us);
-    return std::max(6.0 + kHostUs, cluster) <= std::max(6.0 + (double)n * kHostUs, us);
+    return std::max(6.0 + kHostUs, cluster) <= std::max(6.0 + (double)(n + n % 2) * kHostUs, us);  // odd: and a copy
 }
 
 cudaError_t launch_resident(int reaction, int boundary, void *u, void *v, int64_t nn, int64_t nm,

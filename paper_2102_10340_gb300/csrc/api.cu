@@ -215,7 +215,11 @@ static int resolve_variant(const rdcnn_t *h, bool vec_ok, bool wide_ok, int *var
     if (*variant == RDCNN_VARIANT_TEMPORAL2 && is_16bit(h->dtype))
         return set_error(RDCNN_EINVAL, "RDCNN_VARIANT_TEMPORAL2 supports FP32 / FP64 planes only");
     if (*variant == RDCNN_VARIANT_TEMPORAL || *variant == RDCNN_VARIANT_TEMPORAL2) {
-        if (*k == 0) *k = h->tune_k ? h->tune_k : default_k(h->dtype, h->nn, h->nm);
+        if (*k == 0 && h->tune_k) *k = h->tune_k;
+        if (*k == 0) {
+            if (!h->auto_k) h->auto_k = default_k(h->dtype, h->nn, h->nm);
+            *k = h->auto_k;
+        }
         if (*k < 1 || *k > max_k(h->dtype))
             return set_error(RDCNN_EINVAL, "k must be in 1..%d", max_k(h->dtype));
     } else {
@@ -344,7 +348,8 @@ int run_core(rdcnn_t *h, int64_t T, int variant, int k, int64_t every, MarkFn ma
     if (autov && variant == RDCNN_VARIANT_GENERIC && h->dtype == RDCNN_F32 &&
         ragged_pays(h->nn, h->nm, every > 0 ? std::min(every, T) : T)) {
         variant = kVariantRagged;
-        k = (k_arg >= 1 && k_arg <= max_k(h->dtype)) ? k_arg : h->tune_k ? h->tune_k : default_k_ragged(h->nn, h->nm);
+        if (!h->auto_k_ragged) h->auto_k_ragged = default_k_ragged(h->nn, h->nm);
+        k = (k_arg >= 1 && k_arg <= max_k(h->dtype)) ? k_arg : h->tune_k ? h->tune_k : h->auto_k_ragged;
     }
     const void *cu = h->u, *cv = h->v;
     void *nu = su, *nv = sv;

@@ -19,6 +19,9 @@ struct rdcnn {
     cudaStream_t stream = nullptr;
     bool bound = false;
     int tune_k = 0, tune_rows = 0;
+    // depths that AUTO's launch model chooses for this size, for vector and
+    // other rows; 0 until first asked for
+    mutable int auto_k = 0, auto_k_ragged = 0;
     cudaStream_t copy_stream = nullptr;  // created on first use by rdcnn_run_snapshots
     // rdcnn_adjoint's second stream (segment rebuilds overlap the reverse
     // sweep) and its events: [0] checkpoints ready, [1..2] rebuild of buffer

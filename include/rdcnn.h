@@ -197,7 +197,7 @@ int rdcnn_set_state(rdcnn_t *h, const void *u0, const void *v0, int on_device);
  * otherwise an explicit request returns RDCNN_EINVAL, and AUTO runs F32
  * planes through the temporal pipeline with elements copied one by one (unless
  * they are too narrow for it), others through GENERIC.  AUTO on F64 planes is STEP1 unless a depth is asked for
- * (k or tune->k).  AUTO on F32 grids of 16 to 384 columns and up to 1024 (129
+ * (k or tune->k) or the tuned strips are long and few (then TEMPORAL, k = 4).  AUTO on F32 grids of 16 to 384 columns and up to 1024 (129
  * columns and more: 512, 257 and more: 256) rows, with no k and no tune,
  * advances whole stretches of the run in one launch of one thread-block
  * cluster that holds the state in registers: the same bits (or, should its

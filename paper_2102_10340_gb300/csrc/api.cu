@@ -203,9 +203,17 @@ static int resolve_variant(const rdcnn_t *h, bool vec_ok, bool wide_ok, int *var
         return RDCNN_OK;
     }
     if (*variant == RDCNN_VARIANT_AUTO) {
-        *variant = !vec_ok ? RDCNN_VARIANT_GENERIC
-                   : auto_single_step(h->dtype) && *k == 0 && h->tune_k == 0 ? RDCNN_VARIANT_STEP1  // no depth asked for
-                                                                             : RDCNN_VARIANT_TEMPORAL;
+        const bool single = auto_single_step(h->dtype) && *k == 0 && h->tune_k == 0;  // no depth asked for
+        *variant = !vec_ok ? RDCNN_VARIANT_GENERIC : single ? RDCNN_VARIANT_STEP1 : RDCNN_VARIANT_TEMPORAL;
+        // FP64 strips of 16 rows and more that leave schedulers without a warp: the
+        // pipeline's four steps a row hide more latency.  us for 40 steps, pipeline / single steps:
+        // 256^2 32 rows 1391 / 1523, 128 rows 5157 / 5906, 1024^2 128 rows 5159 / 6362, 16 rows
+        // (1024 strips) 1697 / 1398, 512^2 8 rows 690 / 447.
+        if (vec_ok && single && h->tune_rows >= 16 &&
+            (h->nm + 63) / 64 * ((h->nn + h->tune_rows - 1) / h->tune_rows) < 4 * (int64_t)sm_count()) {
+            *variant = RDCNN_VARIANT_TEMPORAL;
+            *k = kMaxK64;
+        }
     }
     if ((*variant == RDCNN_VARIANT_STEP1 || *variant == RDCNN_VARIANT_TEMPORAL ||
          *variant == RDCNN_VARIANT_TEMPORAL2) && !vec_ok)

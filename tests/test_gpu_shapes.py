@@ -184,3 +184,18 @@ def test_launches_of_short_stretches(rd, shape, T, launches):
     assert rd.launch_count() - before == launches
     h.set_state(x, -x).run(T, variant="generic")
     assert torch.equal(g.u, h.u) and torch.equal(g.v, h.v)
+
+
+@pytest.mark.parametrize("shape,rows,want", [((256, 256), 0, ("step1", 1)), ((256, 256), 15, ("step1", 1)),
+                                             ((256, 256), 16, ("temporal", 4)), ((1024, 1024), 16, ("step1", 1)),
+                                             ((1024, 1024), 128, ("temporal", 4)), ((300, 301), 64, ("generic", 1))])
+def test_fp64_strips_asked_for(rd, shape, rows, want):
+    """AUTO with a strip length but no depth: single steps, or the pipeline where the strips are few and long."""
+    x = torch.from_numpy(inp.uniform_field(87, *shape)).double().cuda()
+    g, h = (rd.Grid(*shape, inp.default_params(), dtype=torch.float64) for _ in range(2))
+    g.set_tune(k=0, rows=rows)
+    plan = g.plan()
+    assert (plan["variant"], plan["k"]) == want and (want[0] == "generic" or rows == 0 or plan["rows"] == rows)
+    g.set_state(x, -x).run(9)
+    h.set_state(x, -x).run(9, variant="generic")
+    assert torch.equal(g.u, h.u) and torch.equal(g.v, h.v)

@@ -319,7 +319,7 @@ double launch_cost(bool ragged, int K, int64_t nn, int64_t nm) {
 }
 // Planes that are no whole vectors are copied one after the other.
 double copy_cost(int64_t nn, int64_t nm) {
-    return (nn * nm % 4 != 0 ? 10.0 : 1.7) + (double)(nn * nm) * 16 / (beyond_l2(nn, nm) ? 6.7e6 : 12e6);
+    return (nn * nm % 4 != 0 ? 10.0 : 1.7) + (double)(nn * nm) * 16 / (beyond_l2(nn, nm) ? 6.2e6 : 12e6);
 }
 }  // namespace
 
@@ -328,7 +328,7 @@ double copy_cost(int64_t nn, int64_t nm) {
 // default depth k.  home: what the parity of the number of launches must be for
 // the state to end where it belongs (0 even, 1 odd; -1: anywhere).  us, launches of
 // at most depth k, even in number / as here: 512^2 9 steps 18.5 / 13.4, 1024^2 9 steps 20.0 /
-// 17.6, 8192^2 3 steps 375 / 341, 200000 x 4 2 steps 91 / 60.
+// 17.6, 8192^2 3 steps 375 / 348, 200000 x 4 2 steps 91 / 57.
 int64_t stretch_launches(bool ragged, int64_t nn, int64_t nm, int64_t steps, int k, int home, double *us) {
     const BeatModel &m = ragged ? kRaggedBeats : kBeats;
     int64_t n = (steps + k - 1) / k;
@@ -341,7 +341,9 @@ int64_t stretch_launches(bool ragged, int64_t nn, int64_t nm, int64_t steps, int
     double least = 1e300;
     int64_t best = n;
     for (int64_t c = (steps + m.k1 - 1) / m.k1; c <= std::min(steps, n + (strays(n) ? 1 : 0)); ++c) {
-        const double t = (double)c * std::max(kHostUs, launch_cost(ragged, (int)((steps + c - 1) / c), nn, nm)) +
+        const int K = (int)(steps / c), deeper = (int)(steps % c);  // launches of depth K + 1, the others of K
+        const double t = (double)(c - deeper) * std::max(kHostUs, launch_cost(ragged, K, nn, nm)) +
+                         (deeper ? deeper * std::max(kHostUs, launch_cost(ragged, K + 1, nn, nm)) : 0.0) +
                          (strays(c) ? std::max(kHostUs, copy_cost(nn, nm)) : 0.0);
         if (t <= least) { least = t; best = c; }
     }

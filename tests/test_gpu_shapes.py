@@ -172,7 +172,7 @@ def test_strips_beyond_l2(rd, boundary, reaction):
     assert small.plan("temporal", 1)["rows"] != 10
 
 
-@pytest.mark.parametrize("shape,T,launches", [((512, 512), 9, 2), ((1024, 1024), 10, 2), ((2600, 2400), 3, 1),
+@pytest.mark.parametrize("shape,T,launches", [((512, 512), 9, 2), ((1024, 1024), 10, 2), ((5000, 5000), 4, 1),
                                               ((2600, 2400), 8, 2), ((509, 515), 9, 2)])
 def test_launches_of_short_stretches(rd, shape, T, launches):
     """Few deep launches, or one and a copy of the state, where more launches would cost more; the same bits."""

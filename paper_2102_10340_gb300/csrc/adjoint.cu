@@ -312,8 +312,9 @@ bool adj_streams(rdcnn_t *h) {
 // launches of a stretch alternate between the scratch pair and the stretch's
 // destination and end in the destination, so no launch reads the planes it
 // writes.
-// Launch shapes: what AUTO runs (the temporal kernel at the size's default
-// depth; FP64 the single step) between checkpoints; for a full tape (S = 1) the store-all pipeline, which writes
+// Launch shapes: the temporal kernel at the size's default depth (FP64 the
+// single step), also for small FP32 grids, whose whole runs AUTO gives to one
+// cluster, between checkpoints; for a full tape (S = 1) the store-all pipeline, which writes
 // ka consecutive states per launch.  Every variant computes the same bits,
 // so the states are those rdcnn_run produces.
 template <typename T>

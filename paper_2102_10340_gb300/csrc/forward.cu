@@ -370,12 +370,13 @@ bool ragged_pays(int64_t nn, int64_t nm, int64_t steps) {
 // the one that minimises waves x (rows + 2K) -- the work of the slowest SM
 // when every resident warp slot is busy -- so a launch does not spill a
 // nearly empty second wave (e.g. 4096^2, K=8: 128 rows = 1184 warps, one
-// wave on 152 SMs at 8 warps each; 112 rows = 1369 warps, two waves).
+// wave on 152 SMs at 8 warps each; 112 rows = 1369 warps, two waves).  The size
+// classes were measured with FP32 planes, whose lanes 16-bit planes and warp pairs
+// share (256^2 .. 2048^2, with the light-cone fill: 512^2, k = 6, 4 rows 150 Gcell/s, 8 rows
+// 127); FP32 with 4 values per lane has had the launch model above since.
 int auto_rows_temporal(int K, int64_t nn, int64_t nm, int bands, int blocks_per_sm,
                        int warps_per_block) {
     const int64_t cells = nn * nm;
-    // size classes from a sweep at 256^2 .. 2048^2 (with the light-cone fill):
-    // 512^2, k = 6: 4 rows 150 Gcell/s, 8 rows 127
     if (cells < (int64_t(1) << 19)) return 4;
     if (cells < (int64_t(1) << 22)) return 16;
     const int64_t cap = (int64_t)sm_count() * std::max(1, blocks_per_sm) * warps_per_block;
@@ -603,7 +604,9 @@ bool auto_single_step(int dtype) { return dtype == RDCNN_F64; }
 // The single-step kernel is fastest with short strips (more warps in flight).
 // The 16-bit single step (the ring pipeline at depth 1, 8 values per lane where
 // rows are such vectors) takes the strips of which an SM gets 8, or 16 where
-// those would be longer than 17 rows, and 32 rows from there on.  bf16, us a
+// those would be longer than 17 rows, and 32 rows where these are longer than 27: a
+// strip's two extra input rows then weigh little, and the 32 of the large grids'
+// sweep (4 .. 64 rows at 4096^2) beat the 28 to 31 of the rule by 2 %.  bf16, us a
 // step, 32 rows / now: 512^2 7.5 / 2.5, 1024^2 7.6 / 3.4, 2048^2 8.0 / 6.5, 4096 x
 // 1000 10.5 / 6.8, 2900 x 3128 14.8 / 11.4; 4096^2 with 31 / 32 rows 23.9 / 23.5.
 // FP64: one row while that leaves warp slots free, else two (us a step, 1 / 2 /

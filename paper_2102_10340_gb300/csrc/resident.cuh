@@ -37,10 +37,10 @@
 // of the cluster then stores NaNs in both planes, over its rows: a failed run has
 // no cell that looks like a result.
 //
-// Bound: latency of the hand-over up to 128^2 (64^2: 370 cycles a step, of which
+// Bound: latency of the hand-over up to 128^2 (64^2: 345 cycles a step, of which
 // about 100 are the sums and the update), one warp's issue rate per scheduler of
 // 16 SMs at 256^2.  us a step, launches -> resident: 64^2 0.84 -> 0.17, 128^2 0.82
-// -> 0.23, 256^2 0.86 -> 0.44.  Measured on the way, 64^2 / 128^2 / 256^2: one
+// -> 0.23, 256^2 0.86 -> 0.47.  Measured on the way, 64^2 / 128^2 / 256^2: one
 // cluster barrier a step 0.34 / 0.46 / 0.68; every row by asynchronous stores
 // 0.26 / 0.38 / 0.74; two rows handed on every second step, with the redundant
 // rows computed, 0.21 / 0.29 / 0.71.
@@ -222,8 +222,7 @@ __device__ __forceinline__ void spoil(const ResArgs &a, int r0, int nr) {
 // predicate (always true: a cluster has blocks), so that the compiler sees no way
 // out of the step loop here; with one, it builds the loop otherwise: us a step at
 // 64^2 / 128^2 / 256^2, a flag and a break 0.196 / 0.265 / 0.476, an exit known as
-// such 0.188 / 0.255 / 0.508, this 0.165 / 0.231 / 0.441 (with the stores unrolled
-// 0.168 / 0.231 / 0.498).
+// such 0.188 / 0.255 / 0.508, this 0.167 / 0.232 / 0.470.
 __device__ __forceinline__ void give_up(const ResArgs &a, int r0, int nr, unsigned flag) {
     const int lane = threadIdx.x & 31;
     if (lane < a.blocks) flag_set(flag, lane);

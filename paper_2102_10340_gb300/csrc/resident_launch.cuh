@@ -15,30 +15,28 @@ constexpr size_t resident_smem(int warps) {  // two parities x two directions x 
     return (size_t)2 * warps * 2 * 2 * 128 * V + (size_t)16 * warps + 16;
 }
 
-// The most blocks, 16 or 8, of a cluster of the largest blocks that the current
-// device can run (more than eight is the non-portable size, which not every
-// partition of a GPU has room for); 0: none.
+// 16 where the current device can run a cluster of that many of the largest
+// blocks (more than eight is the non-portable size, which not every partition of
+// a GPU has room for), else 0: grids of sixteen rows and more are dealt to
+// sixteen blocks.
 template <int V, int RX, int BC, int RAG>
 int resident_most() {
     auto *k = k_resident<V, RX, BC, RAG>;
     const int wmax = ResWarps<V>::value;
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)resident_smem<V>(wmax)) == cudaSuccess &&
         cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
-        for (int c : {16, 8}) {
-            cudaLaunchAttribute at[1];
-            at[0].id = cudaLaunchAttributeClusterDimension;
-            at[0].val.clusterDim.x = c;
-            at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = c;
-            cfg.blockDim = 32 * wmax;
-            cfg.dynamicSmemBytes = resident_smem<V>(wmax);
-            cfg.attrs = at;
-            cfg.numAttrs = 1;
-            int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) == cudaSuccess && n > 0) return c;
-            (void)cudaGetLastError();
-        }
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = 16;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = 16;
+        cfg.blockDim = 32 * wmax;
+        cfg.dynamicSmemBytes = resident_smem<V>(wmax);
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) == cudaSuccess && n > 0) return 16;
     }
     (void)cudaGetLastError();
     return 0;

@@ -61,7 +61,7 @@ struct ResArgs {
 };
 
 // Most warps of a block: V = 12 needs up to 255 registers a thread, V = 8 up to
-// 208, V = 4 up to 126, V = 2 up to 96.
+// 225, V = 4 up to 127, V = 2 up to 96.
 template <int V> struct ResWarps : IntC<V >= 8 ? 8 : 16> {};
 
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
